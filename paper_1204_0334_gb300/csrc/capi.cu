@@ -1,5 +1,5 @@
 // C-ABI entry points of the block-code decoder (include/ldpc.h).
-#include "ldpc_internal.cuh"
+#include "flow_internal.cuh"
 
 #include <algorithm>
 #include <chrono>
@@ -211,6 +211,7 @@ ldpc_status ldpc_code_destroy(ldpc_code c) {
     cudaFree(w.stage_hard);
     cudaFree(w.stage_i32);
     noms_free(c->noms);
+    flow_free(c->flow);
     sim_free(c->sim);
     enc_free(c->enc);
     cudaFree(c->sp_mem);
@@ -375,8 +376,10 @@ ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc
     const bool host_in = pointer_kind(llr) == 1;
     const bool host_out = (post && pointer_kind(post) == 1) || (hard && pointer_kind(hard) == 1) ||
                           (iters && pointer_kind(iters) == 1) || (ok && pointer_kind(ok) == 1);
-    st = qc_ensure_workspace(c, (size_t)gamma, host_in || host_out);
-    if (st != LDPC_OK) return st;
+    if (host_in || host_out) {
+        st = qc_ensure_stage(c, (size_t)gamma);
+        if (st != LDPC_OK) return st;
+    }
     DecodeWs &w = c->ws;
     const size_t NB = (size_t)gamma * c->d.N;
     const float *src = llr;
@@ -384,16 +387,23 @@ ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc
         LDPC_CUDA_TRY(cudaMemcpyAsync(w.stage_llr, llr, NB * 4, cudaMemcpyHostToDevice, s));
         src = w.stage_llr;
     }
-    st = qc_pack_llr(c, src, gamma, o, s);
-    if (st != LDPC_OK) return st;
-    st = qc_decode_device(c, gamma, o, post != nullptr, s);
-    if (st != LDPC_OK) return st;
     float *d_post = post && pointer_kind(post) == 1 ? w.stage_post : post;
     uint8_t *d_hard = hard && pointer_kind(hard) == 1 ? w.stage_hard : hard;
     int32_t *d_iters = iters && pointer_kind(iters) == 1 ? w.stage_i32 : iters;
-    int32_t *d_ok = ok && pointer_kind(ok) == 1 ? w.stage_i32 + w.gamma_cap : ok;
-    st = qc_unpack_outputs(c, gamma, o, d_post, d_hard, d_iters, d_ok, s);
-    if (st != LDPC_OK) return st;
+    int32_t *d_ok = ok && pointer_kind(ok) == 1 ? w.stage_i32 + w.stage_cap : ok;
+    if (!c->sparse && flow_pays(c->d, gamma, o)) {
+        st = flow_decode_code(c, src, gamma, o, d_post, d_hard, d_iters, d_ok, s);
+        if (st != LDPC_OK) return st;
+    } else {
+        st = qc_ensure_workspace(c, (size_t)gamma);
+        if (st != LDPC_OK) return st;
+        st = qc_pack_llr(c, src, gamma, o, s);
+        if (st != LDPC_OK) return st;
+        st = qc_decode_device(c, gamma, o, post != nullptr, s);
+        if (st != LDPC_OK) return st;
+        st = qc_unpack_outputs(c, gamma, o, d_post, d_hard, d_iters, d_ok, s);
+        if (st != LDPC_OK) return st;
+    }
     if (d_post != post) LDPC_CUDA_TRY(cudaMemcpyAsync(post, d_post, NB * 4, cudaMemcpyDeviceToHost, s));
     if (d_hard != hard) LDPC_CUDA_TRY(cudaMemcpyAsync(hard, d_hard, NB, cudaMemcpyDeviceToHost, s));
     if (d_iters != iters) LDPC_CUDA_TRY(cudaMemcpyAsync(iters, d_iters, (size_t)gamma * 4, cudaMemcpyDeviceToHost, s));
@@ -416,7 +426,7 @@ ldpc_status ldpc_channel(ldpc_code c, double ebn0_db, uint64_t seed, uint64_t fi
     const bool host_out = pointer_kind(llr_out) == 1;
     float *dst = llr_out;
     if (host_out) {
-        ldpc_status st = qc_ensure_workspace(c, (size_t)gamma, 1);
+        ldpc_status st = qc_ensure_stage(c, (size_t)gamma);
         if (st != LDPC_OK) return st;
         dst = c->ws.stage_llr;
     }

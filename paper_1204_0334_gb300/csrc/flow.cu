@@ -1,0 +1,291 @@
+// The flow decoder: Algorithm 1 on a batch of frames in one persistent launch.
+//
+// A decode as a sequence of launches (check pass, variable pass, syndrome, list of running
+// packages, thirty times) streams the whole message store through HBM in every pass, leaves the
+// chip idle between passes, and launches all iterations whether or not a frame still runs.  Here
+// blocks work through tiles: a tile is a few check rows of one package, a few variables, some rows
+// of its syndrome, or a piece of the transposes in and out.
+//
+//  * W packages are in work at a time, each in a slot with its own message, channel-LLR and decision
+//    buffers; W is chosen so that the slots' buffers stay in L2, where an in-place copy runs at
+//    6.2 TB/s each way against 3.3 through HBM.  A slot whose package is finished takes the next one.
+//  * A slot is in one phase: pack the LLRs, check step, variable step, syndrome, output.  Whoever
+//    finishes the last tile of a phase opens the slot's next phase: it appends an entry to a log that
+//    every block reads.  An entry says how many tiles were opened before it, and tile i of it goes to
+//    block (that + i) mod blocks, so the blocks share the tiles evenly without an atomic per tile
+//    (handing tiles out by atomics: 3200 cycles a tile in the block's serial part).  With several
+//    packages in work the chip stays full through phase ends, and a package stops the moment its
+//    frames have.
+//  * No tile waits for another: a block that has a tile always finishes it, so any number of resident
+//    blocks makes progress on the tiles that are theirs; all of a launch's blocks are resident (one an
+//    SM).  Every wait has a limit, after which the launch ends and the object reports a timeout.
+//  * Within a block, one warp reads the log and starts the bulk copies of its tiles' lines (the rows
+//    of a tile meet each circulant in one run of consecutive edges, or two at its wrap: a copy and an
+//    address per slot of all the tile's rows, not per edge); 24 warps compute out of shared memory and
+//    in place (a row, or a variable, per warp, a frame, or two, or four, per lane); a warp per stage
+//    stores the results by bulk copies and counts the tile done once they have landed.
+//
+// Three stages of 72 KB: a tile arrives while another is computed and a third leaves.  What bounds it
+// (n = 18360, FP32, 2048 frames, 30 iterations): the compute warps, 5500 cycles a check tile and 3600
+// a variable tile of the 5400 a tile takes on average (about 50 instructions per edge and iteration,
+// 81 in the launches before).  15.2 ms before, 11.2 ms now; the n = 15168 integer min-sum with early
+// stop, 4096 frames: 3.17 -> 2.00 ms; 40 frames of the n = 18360 code with early stop: 749 -> 267 us
+// (the launches of all 30 iterations are gone); an irregular n = 2532 code, 1000 frames: 886 -> 377 us.
+//
+// The arithmetic is that of the pass kernels (qc_pipe.cu), operation by operation.
+#include "flow_internal.cuh"
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <mutex>
+#include <new>
+#include <unordered_map>
+
+namespace ldpc {
+namespace flow {
+
+int resident_blocks(const void *kernel, size_t smem) {
+    static std::mutex mu;
+    static std::unordered_map<const void *, int> blocks;
+    std::lock_guard<std::mutex> lk(mu);
+    auto f = blocks.find(kernel);  // each kernel has one shared-memory size
+    if (f != blocks.end()) return f->second;
+    int dev = 0, sms = 0, bps = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, kThreads, smem);
+    cudaGetLastError();
+    return blocks[kernel] = bps * sms;
+}
+
+// rows and variables of a tile by the code's degrees and the storage (as Cfg in flow.cuh)
+static void tile_sizes(const QcDesc &d, int FV, int *rows, int *rows1, int *kc) {
+    *rows = tile_rows(d.J, d.L);
+    *rows1 = *rows / FV;
+    *kc = d.J <= 4 ? 4 * kComputeWarps : 2 * kComputeWarps;
+}
+
+static uint32_t fill_code(const QcDesc &d, int FV, Code &c) {
+    std::memset(&c, 0, sizeof(c));
+    int rows, rows1, kc;
+    tile_sizes(d, FV, &rows, &rows1, &kc);
+    c.J = d.J, c.L = d.L, c.p = d.p, c.N = d.N, c.M = d.M;
+    // tiles of equal size within a column, in multiples of four variables
+    const int vch = (d.p + kc - 1) / kc;
+    c.kc = std::min(kc, ((d.p + vch - 1) / vch + 3) / 4 * 4);
+    c.nsyn = (d.M + kComputeWarps * 32 - 1) / (kComputeWarps * 32);
+    c.divp = fast_div((uint32_t)d.p);
+    c.rch = fast_div((uint32_t)((d.p + rows - 1) / rows));
+    c.rch1 = fast_div((uint32_t)((d.p + rows1 - 1) / rows1));
+    c.vch = fast_div((uint32_t)((d.p + c.kc - 1) / c.kc));
+    std::memcpy(c.sh, d.shift, sizeof(int) * d.J * d.L);
+    std::memcpy(c.eo, d.eoff, sizeof(int) * d.J * d.L);
+    return std::max(c.J * c.rch1.d + (uint32_t)c.nsyn, c.L * c.vch.d);  // tiles of the largest phase
+}
+
+// the code table's entry, an empty log, every slot with its first package and its pack phase open
+__global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args a) {
+    const int *src = reinterpret_cast<const int *>(&st.code);
+    int *dst = reinterpret_cast<int *>(a.codes);
+    const int V = st.V;
+    for (int i = threadIdx.x; i < (int)(sizeof(Code) / 4); i += blockDim.x) dst[i] = src[i];
+    if (threadIdx.x == 0) {
+        a.ctl->tail = ((unsigned long long)a.W << 40) | ((unsigned long long)a.W * st.tiles);
+        a.ctl->next = a.W;
+        a.ctl->live = a.W;
+        a.ctl->abort = 0;
+    }
+    for (int n = threadIdx.x; n < kLog; n += blockDim.x) {
+        Entry e;
+        if (n < a.W) {
+            e.w0 = entry_w0(F_PACK, 0, 1, 0, n);
+            e.w1 = entry_w1((uint32_t)n, n, (uint32_t)(((long long)n * st.tiles) % a.blocks), (uint32_t)st.tiles);
+        } else {
+            e.w0 = 0ull;
+            e.w1 = entry_w1((uint32_t)n - kLog, 0, 0u, 0u);  // the sequence number of the lap before
+        }
+        a.log[n] = e;
+    }
+    const int s = threadIdx.x;
+    if (s >= a.W) return;
+    Slot &sl = a.slots[s];
+    sl.all = 0;
+    sl.done = sl.syn_done = 0u;
+    for (int v = 0; v < V; ++v) {
+        uint32_t valid = 0u;
+        for (int ln = 0; ln < 32; ++ln)
+            if ((s * 32 + ln) * V + v < st.code.gamma) valid |= 1u << ln;
+        sl.dn[v] = ~valid;
+        sl.un[v] = 0u;
+    }
+}
+
+ldpc_status start(const Args &a, const Start &st, cudaStream_t s) {
+    start_kernel<<<1, 1024, 0, s>>>(st, a);
+    count_launch();
+    LDPC_CUDA_TRY(cudaGetLastError());
+    return LDPC_OK;
+}
+
+}  // namespace flow
+
+using namespace flow;
+
+size_t flow_ctl_bytes(int W) {
+    return (size_t)W * sizeof(Slot) + 256 + kLog * sizeof(Entry) + sizeof(Code);
+}
+
+void flow_slot_bytes(const QcDesc &d, int msg, int algo, bool post, size_t *b4) {
+    const int V = lanes_per_word(msg), FV = algo == LDPC_ALGO_MS ? 1 : V;
+    b4[0] = (size_t)d.E * 128;
+    b4[1] = (size_t)d.N * 128 * FV;
+    b4[2] = post ? (size_t)d.N * 128 * V : 0;
+    b4[3] = ((size_t)d.N * V * 4 + 127) / 128 * 128;
+}
+
+// L2 the slots' buffers may take: reads of a resident buffer keep their full rate up to about
+// 110 MB on this chip (20 TB/s, 13 at 120 MB, 8 past L2)
+constexpr size_t kL2Budget = (size_t)96 << 20;
+
+int flow_slots(const QcDesc &d, int msg, int algo, bool post, int P) {
+    size_t b[4];
+    flow_slot_bytes(d, msg, algo, post, b);
+    const size_t one = b[0] + b[1] + b[2] + b[3];
+    const size_t fit = kL2Budget / one;
+    return (int)std::min<size_t>({(size_t)P, (size_t)kMaxSlots, std::max<size_t>(fit, 4)});
+}
+
+// A phase of the flow takes 6 us however few its tiles (8 with FP16 or int8 messages), a pass of its
+// own launch 4.5 us: with a fixed iteration count the launches are faster below about 80000 message
+// lines (edges times packages).  20 iterations, launches / flow: n = 384, 32 frames (1152 lines) 205 /
+// 259 us; 4 x 12, p = 211, 256 frames (81024) 419 / 336; 4 x 24, p = 300, 32 frames (28800) 294 / 355,
+// 128 frames (115200) 465 / 394.  Short codes fill a tile badly: 3 x 6, p = 64, 2048 frames (73728)
+// 419 / 572, 4 x 8, p = 100, 2048 frames (204800) 720 / 801.  With early stop the flow ends with the
+// last frame and its syndrome takes no launches, so it is taken unless the code is short and the
+// batch large.
+bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o) {
+    const int W = 32 * lanes_per_word(o.msg);
+    const long long lines = (long long)d.E * ((gamma + W - 1) / W);
+    const bool shortcode = d.E < 8000;
+    return o.early_stop ? !shortcode || lines < 60000 : !shortcode && lines > 80000;
+}
+
+ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int gamma, const ldpc_decode_opts &o,
+                        float *post, uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+    const int V = lanes_per_word(o.msg), FV = o.algo == LDPC_ALGO_MS ? 1 : V;
+    if (m.err && *(volatile int *)m.err) {
+        set_error("an earlier decode of this object gave up a device-side wait (code %d)", *m.err);
+        *m.err = 0;
+        return LDPC_ETIMEOUT;
+    }
+    Start st;
+    Code &c = st.code;
+    const uint32_t tiles = fill_code(d, FV, c);
+    if (tiles >= (1u << kLogTiles) || gamma / (32 * V) >= (1 << kLogPk) || o.max_iter >= (1 << kLogIt)) {
+        set_error("code too long: %u tiles a phase", tiles);
+        return LDPC_EINVAL;
+    }
+    c.gamma = gamma;
+    c.llr = llr, c.post = post, c.hard = hard, c.iters = iters, c.ok = ok;
+    c.nparams = o.algo == LDPC_ALGO_NOMS ? o.noms_params : nullptr;
+    Args a;
+    std::memset(&a, 0, sizeof(a));
+    size_t b[4];
+    flow_slot_bytes(d, o.msg, o.algo, post != nullptr, b);
+    a.slots = (Slot *)m.ctl;
+    a.ctl = (Ctl *)((char *)m.ctl + (size_t)m.W * sizeof(Slot));
+    a.log = (Entry *)((char *)a.ctl + 256);
+    a.codes = (Code *)(a.log + kLog);
+    a.ncodes = 1;
+    a.P = (gamma + 32 * V - 1) / (32 * V);
+    a.W = std::min(m.W, a.P);
+    a.msg = (uint32_t *)m.msg, a.mu = (uint32_t *)m.mu, a.post = (float *)m.post, a.hw = (uint32_t *)m.hw;
+    a.msg_stride = b[0] / 4, a.mu_stride = b[1] / 4, a.post_stride = b[2] / 4, a.hw_stride = b[3] / 4;
+    a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post != nullptr;
+    a.clip = o.clip, a.qscale = ldexpf(1.0f, o.frac_bits), a.lsb = ldexpf(1.0f, -o.frac_bits);
+    a.err = m.err;
+    // with several packages in work a phase of its own for the syndrome costs no time and saves the
+    // check step of a package that has stopped; with few it would add its latency to every iteration
+    a.split = a.early && a.W >= 4;
+    st.V = V;
+    st.tiles = (d.N + outv(d.J) - 1) / outv(d.J);
+    Shape g{d.J, d.L, 1};
+    for (int i = 0; i < d.J * d.L; ++i) g.regular &= d.shift[i] >= 0;
+    const int grid = (int)std::min<long long>((long long)tiles * a.W, 1 << 20);
+    if (o.algo == LDPC_ALGO_MS) return run_ms(a, st, g, grid, s);
+    if (o.algo == LDPC_ALGO_NOMS)
+        return o.msg == LDPC_MSG_F16 ? run_noms16(a, st, g, grid, s) : run_noms32(a, st, g, grid, s);
+    return o.msg == LDPC_MSG_F16 ? run_sp16(a, st, g, grid, s) : run_sp32(a, st, g, grid, s);
+}
+
+}  // namespace ldpc
+
+// ---------------------------------------------------------------------------
+// the workspace a code object keeps
+// ---------------------------------------------------------------------------
+struct ldpc_flow_ws {
+    size_t cap[4] = {0, 0, 0, 0};
+    void *buf[4] = {nullptr, nullptr, nullptr, nullptr};
+    void *ctl = nullptr;
+    int *err = nullptr;  // pinned, device-mapped
+};
+
+namespace ldpc {
+
+void flow_free(ldpc_flow_ws *w) {
+    if (!w) return;
+    for (void *b : w->buf) cudaFree(b);
+    cudaFree(w->ctl);
+    if (w->err) cudaFreeHost(w->err);
+    delete w;
+}
+
+ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
+                             uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+    const int V = lanes_per_word(o.msg);
+    const int W = flow_slots(c->d, o.msg, o.algo, post != nullptr, (gamma + 32 * V - 1) / (32 * V));
+    auto fail = [&](size_t bytes) {
+        cudaGetLastError();
+        set_error("device allocation of the decoder's workspace (%zu bytes) failed", bytes);
+        return LDPC_ENOMEM;
+    };
+    if (!c->flow) {
+        c->flow = new (std::nothrow) ldpc_flow_ws();
+        if (!c->flow) return fail(0);
+    }
+    ldpc_flow_ws &w = *c->flow;
+    if (!w.ctl && cudaMalloc(&w.ctl, flow_ctl_bytes(kMaxSlots)) != cudaSuccess) {
+        w.ctl = nullptr;
+        return fail(flow_ctl_bytes(kMaxSlots));
+    }
+    if (!w.err) {
+        if (cudaHostAlloc((void **)&w.err, 64, cudaHostAllocMapped) != cudaSuccess) {
+            w.err = nullptr;
+            return fail(64);
+        }
+        *w.err = 0;
+    }
+    size_t b[4];
+    flow_slot_bytes(c->d, o.msg, o.algo, post != nullptr, b);
+    bool synced = false;
+    for (int i = 0; i < 4; ++i) {
+        const size_t need = b[i] * W;
+        if (need <= w.cap[i]) continue;
+        if (!synced) LDPC_CUDA_TRY(cudaDeviceSynchronize());
+        synced = true;
+        cudaFree(w.buf[i]);
+        w.buf[i] = nullptr;
+        w.cap[i] = 0;
+        if (cudaMalloc(&w.buf[i], need) != cudaSuccess) {
+            w.buf[i] = nullptr;
+            return fail(need);
+        }
+        w.cap[i] = need;
+    }
+    FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.err};
+    return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
+}
+
+}  // namespace ldpc

@@ -1,0 +1,139 @@
+// Shared declarations of the flow decoder (flow.cu describes it).
+#pragma once
+
+#include "ldpc_internal.cuh"
+
+namespace ldpc {
+namespace flow {
+
+// One block per SM.  24 compute warps leave 72 registers a thread; with 16 (96 registers) the
+// 2048-frame decode of the n = 18360 code took 19.2 ms where 24 took 14.9 (before the other steps):
+// the rows are chains of dependent instructions, and warps hide them better than registers.
+constexpr int kComputeWarps = 24;
+constexpr int kStages = 3;                          // tiles a block holds: in work, arriving, leaving
+constexpr int kThreads = (kComputeWarps + 1 + kStages) * 32;  // and the taking warp, a retiring warp per stage
+constexpr int kLookLimit = 1 << 24;                 // looks for a new phase before a block gives up (seconds)
+constexpr int kMaxSlots = 256;
+constexpr int kLog = 4096;                          // entries of the phase log (a power of two)
+// check rows of a tile: one a compute warp (two of short rows; fewer of 32-edge rows, so that three
+// tiles fit in shared memory)
+__host__ __device__ constexpr int tile_rows(int J, int L) {
+    return J <= 4 && L <= 8 ? 2 * kComputeWarps : (L <= 24 ? kComputeWarps : kComputeWarps * 2 / 3 / 2 * 2);
+}
+__host__ __device__ constexpr int outv(int J) { return J <= 4 ? 256 : 128; }  // variables of a pack / output tile
+static_assert(kComputeWarps % 2 == 0, "row, frame pairs of the first iteration");
+
+enum { kFlowSP = 0, kFlowMS = 1, kFlowNOMS = 2 };
+enum { F_PACK = 0, F_CN, F_VN, F_FIN, F_OUT, F_SYN, F_EXIT };  // phases; F_SYN: also a tile of F_CN and F_FIN
+
+// one code of a flow and the caller's buffers of its frames
+struct Code {
+    int J, L, p, N, M;
+    int kc;                  // variables of a variable tile (a multiple of 4)
+    int nsyn;                // syndrome tiles
+    FastDiv divp, rch, rch1, vch;  // p; check tiles per block row (later / first iteration); variable tiles per column
+    int pk0, gamma;          // first package of the flow that is this code's, frames
+    const float *llr;
+    float *post;
+    uint8_t *hard;
+    int32_t *iters, *ok;
+    const float *nparams;
+    int sh[kMaxJ * kMaxL], eo[kMaxJ * kMaxL];  // [J][L]: shift (-1: zero block), first edge
+};
+
+// A phase that has been opened, 16 bytes written and read at once.  w0: kind (3 bits), frames stopped
+// (1), iteration (17), code (12), package (26).  w1: tiles (24), the number of tiles opened before it
+// modulo the blocks (10), slot (8), sequence number (22).
+constexpr int kLogIt = 17, kLogCode = 12, kLogPk = 26, kLogTiles = 24, kLogBase = 10, kLogSlot = 8, kLogSeq = 22;
+struct alignas(16) Entry {
+    unsigned long long w0, w1;
+};
+__host__ __device__ inline unsigned long long entry_w0(int kind, int stop, int it, int code, int pk) {
+    unsigned long long x = (unsigned)pk;
+    x = x << kLogCode | (unsigned)code;
+    x = x << kLogIt | (unsigned)it;
+    x = x << 1 | (unsigned)stop;
+    return x << 3 | (unsigned)kind;
+}
+__host__ __device__ inline unsigned long long entry_w1(uint32_t seq, int slot, uint32_t base, uint32_t tiles) {
+    unsigned long long x = seq & ((1u << kLogSeq) - 1u);
+    x = x << kLogSlot | (unsigned)slot;
+    x = x << kLogBase | base;
+    return x << kLogTiles | tiles;
+}
+
+// a package in work
+struct alignas(64) Slot {
+    unsigned int done, syn_done;  // finished tiles of the open phase, finished syndrome tiles
+    int all;                      // every frame has stopped
+    uint32_t dn[4], un[4];        // stopped frames, unsatisfied frames (bit = lane)
+};
+
+struct Ctl {
+    unsigned long long tail;  // phases opened (24 bits), tiles opened (40)
+    int next;                 // packages handed to slots so far
+    int live;                 // slots with a package
+    int abort;                // a wait ran out
+};
+
+struct Args {
+    Code *codes;
+    int ncodes;
+    Slot *slots;
+    Ctl *ctl;
+    Entry *log;
+    int W, P;                  // slots, packages
+    uint32_t *msg, *mu, *hw;   // per slot: [E][32], [N][32 FV], [N][V]
+    float *post;               // per slot: [N][32 V]
+    size_t msg_stride, mu_stride, hw_stride, post_stride;  // words
+    int max_iter, early, want_post;
+    int split;                 // the early-stop syndrome is a phase of its own
+    int blocks;
+    float clip, qscale, lsb;
+    const int *pkg_code;       // package -> code (NULL: one code)
+    int *err;                  // host word set when a wait ran out
+};
+
+struct Shape {
+    int J, L, regular;
+};
+
+// resident blocks of a kernel with kThreads threads (cached per kernel and size)
+int resident_blocks(const void *kernel, size_t smem);
+
+// one translation unit per rule
+// (start: the launch that opens the first phases, once the number of blocks is known)
+struct Start {
+    Code code;
+    int V, tiles;  // lane words' frames; tiles of the pack phase
+};
+ldpc_status run_sp32(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
+ldpc_status run_sp16(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
+ldpc_status run_ms(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
+ldpc_status run_noms32(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
+ldpc_status run_noms16(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
+ldpc_status start(const Args &a, const Start &st, cudaStream_t s);
+
+}  // namespace flow
+
+// the buffers of a flow decode
+struct FlowMem {
+    void *msg, *mu, *post, *hw;  // W slots each
+    void *ctl;                   // flow_ctl_bytes()
+    int W;
+    int *err;
+};
+size_t flow_ctl_bytes(int W);
+// slots a decode of P packages keeps in work, and the bytes of one slot's buffers
+int flow_slots(const QcDesc &d, int msg, int algo, bool post, int P);
+void flow_slot_bytes(const QcDesc &d, int msg, int algo, bool post, size_t *b4);
+// whether a decode goes to the flow decoder rather than to a launch per pass
+bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o);
+// Algorithm 1 on gamma frames of a QC code, device buffers in and out (outputs may be NULL)
+ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int gamma, const ldpc_decode_opts &o,
+                        float *post, uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
+// the same on a code object, in a workspace that it keeps
+ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
+                             uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
+
+}  // namespace ldpc

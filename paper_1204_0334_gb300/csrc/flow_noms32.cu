@@ -1,0 +1,12 @@
+// The flow decoder's kernels: learned min-sum, FP32 messages.
+#include "flow.cuh"
+
+namespace ldpc {
+namespace flow {
+
+ldpc_status run_noms32(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s) {
+    return dispatch<1, kFlowNOMS>(a, st, g, tiles, s);
+}
+
+}  // namespace flow
+}  // namespace ldpc

@@ -1,0 +1,12 @@
+// The flow decoder's kernels: sum-product, FP16 messages.
+#include "flow.cuh"
+
+namespace ldpc {
+namespace flow {
+
+ldpc_status run_sp16(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s) {
+    return dispatch<2, kFlowSP>(a, st, g, tiles, s);
+}
+
+}  // namespace flow
+}  // namespace ldpc

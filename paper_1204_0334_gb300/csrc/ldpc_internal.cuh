@@ -61,7 +61,8 @@ struct DecodeWs {
     int32_t *iters = nullptr;  // [gamma_cap] in package order (frame f)
     unsigned long long *counters = nullptr;  // [8] error counters (ber sim)
     int *act = nullptr;        // [1 + P]: count, then the packages with a frame still running
-    // host-buffer staging
+    // host-buffer staging, grown on its own
+    size_t stage_cap = 0;         // frames
     float *stage_llr = nullptr;   // [gamma][N]
     float *stage_post = nullptr;  // [gamma][N]
     uint8_t *stage_hard = nullptr;
@@ -73,6 +74,7 @@ struct DecodeWs {
 struct ldpc_noms_state;  // training state of the learned min-sum (noms.cu)
 struct ldpc_sim_state;   // frame slots of the continuous simulation (sim.cu)
 struct ldpc_encoder_s;   // systematic encoder (encode.cu)
+struct ldpc_flow_ws;     // workspace of the flow decoder (flow.cu)
 
 namespace ldpc {
 // index tables of a general sparse code (device memory): H in compressed-row form with
@@ -93,6 +95,7 @@ struct ldpc_code_s {
     void *sp_mem = nullptr;   // their device allocation
     ldpc_noms_state *noms = nullptr;
     ldpc_sim_state *sim = nullptr;
+    ldpc_flow_ws *flow = nullptr;
     ldpc_encoder_s *enc = nullptr;   // built on first use, under enc_mu
     std::mutex enc_mu;
     std::vector<int> h_rp, h_col;    // sparse code: H in compressed-row form (host copy)
@@ -125,7 +128,8 @@ double channel_sigma(const ldpc_code c, double ebn0_db);
 inline int flags_per_package(int V) { return 5 * V; }
 
 // launchers implemented in qc_decode.cu
-ldpc_status qc_ensure_workspace(ldpc_code c, size_t gamma, int want_host_stage);
+ldpc_status qc_ensure_workspace(ldpc_code c, size_t gamma);
+ldpc_status qc_ensure_stage(ldpc_code c, size_t gamma);  // the device staging of host buffers
 ldpc_status qc_decode_device(ldpc_code c, int gamma, const ldpc_decode_opts &o, bool want_post,
                              cudaStream_t s);
 ldpc_status qc_pack_llr(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, cudaStream_t s);
@@ -138,6 +142,7 @@ ldpc_status qc_syndrome(ldpc_code c, int P, int V, int word, cudaStream_t s);
 
 ldpc_status phi_eval(const float *x, float *y, int n, int variant, cudaStream_t s);
 void noms_free(ldpc_noms_state *w);
+void flow_free(ldpc_flow_ws *w);
 // pipelined node passes (qc_pipe.cu)
 // fresh (continuous simulation, else NULL): per package [2V] words, bits V..2V-1 mark
 // frames that entered their slot this step; their outgoing messages are set to 0

@@ -20,8 +20,9 @@
 // and messages are written before they are read).  Two calls whose GPU work
 // overlaps -- on two streams, or from two threads -- use the same memory and
 // race; serialize them.
-#include "ldpc_internal.cuh"
+#include "flow_internal.cuh"
 
+#include <algorithm>
 #include <cstring>
 #include <mutex>
 
@@ -31,13 +32,18 @@ constexpr size_t kNoallocBytes = (size_t)16 << 20;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
+// the flow decoder's slots and code table (not part of the 16 MiB that bound a request)
+static __device__ __align__(256) unsigned char g_noalloc_ctl[flow::kMaxSlots * sizeof(flow::Slot) + 256 +
+                                                             flow::kLog * sizeof(flow::Entry) + sizeof(flow::Code)];
+
 namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
-void *g_noalloc_ptr[kMaxDevices] = {};
+void *g_noalloc_ptr[kMaxDevices] = {}, *g_noalloc_ctl_ptr[kMaxDevices] = {};
+int *g_noalloc_err[kMaxDevices] = {};  // pinned host words the flow decoder reports to
 
-// device address of the scratch array on the current device (looked up once per device)
-ldpc_status noalloc_base(void **out) {
+// device addresses of the scratch arrays on the current device (looked up once per device)
+ldpc_status noalloc_base(void **out, void **ctl, int **err) {
     int dev = 0;
     LDPC_CUDA_TRY(cudaGetDevice(&dev));
     if (dev < 0 || dev >= kMaxDevices) {
@@ -49,9 +55,16 @@ ldpc_status noalloc_base(void **out) {
         void *p = nullptr;
         cudaError_t e = cudaGetSymbolAddress(&p, g_noalloc_scratch);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_scratch)");
+        e = cudaGetSymbolAddress(&g_noalloc_ctl_ptr[dev], g_noalloc_ctl);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_ctl)");
+        e = cudaHostAlloc((void **)&g_noalloc_err[dev], 64, cudaHostAllocMapped);
+        if (e != cudaSuccess) return cuda_fail(e, "cudaHostAlloc");
+        *g_noalloc_err[dev] = 0;
         g_noalloc_ptr[dev] = p;
     }
     *out = g_noalloc_ptr[dev];
+    *ctl = g_noalloc_ctl_ptr[dev];
+    *err = g_noalloc_err[dev];
     return LDPC_OK;
 }
 
@@ -107,11 +120,24 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
                   (size_t)(128.0 * (double)kNoallocBytes / (double)noalloc_need(c->d, 128, off)));
         return LDPC_EINVAL;
     }
-    void *base_v = nullptr;
-    st = noalloc_base(&base_v);
+    void *base_v = nullptr, *ctl = nullptr;
+    int *err = nullptr;
+    st = noalloc_base(&base_v, &ctl, &err);
     if (st != LDPC_OK) return st;
     noalloc_need(c->d, cap, off);
     unsigned char *base = (unsigned char *)base_v;
+    cudaStream_t s = (cudaStream_t)stream;
+    if (!c->sparse && flow_pays(c->d, gamma, o)) {
+        // the slots' buffers one after another: a slot takes no more than its package's share of the
+        // bytes counted above (the decision words' rounding fits in the iteration counts', not kept here)
+        const int V = lanes_per_word(o.msg);
+        size_t b[4], at[4], x = 0;
+        flow_slot_bytes(c->d, o.msg, o.algo, post != nullptr, b);
+        const int W = std::min((gamma + 32 * V - 1) / (32 * V), flow::kMaxSlots);
+        for (int i = 0; i < 4; ++i) at[i] = x, x += b[i] * W;
+        const FlowMem m{base + at[0], base + at[1], base + at[2], base + at[3], ctl, W, err};
+        return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
+    }
     // A private view of the code object whose workspace points into the scratch.  It
     // carries everything the decode steps read from a code: the QC description, and for
     // a general code the flag and the device index tables (which stay owned by c).  The
@@ -133,7 +159,6 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
     view.ws.iters = (int32_t *)(base + off[5]);
     view.ws.counters = (unsigned long long *)(base + off[6]);
     view.ws.act = (int *)(base + off[7]);
-    cudaStream_t s = (cudaStream_t)stream;
     st = qc_pack_llr(&view, llr, gamma, o, s);
     if (st != LDPC_OK) return st;
     st = qc_decode_device(&view, gamma, o, post != nullptr, s);

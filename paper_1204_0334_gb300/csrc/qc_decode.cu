@@ -423,55 +423,67 @@ ldpc_status phi_eval(const float *x, float *y, int n, int variant, cudaStream_t 
 // ---------------------------------------------------------------------------
 static size_t round_up(size_t x, size_t a) { return (x + a - 1) / a * a; }
 
-ldpc_status qc_ensure_workspace(ldpc_code c, size_t gamma, int want_host_stage) {
+ldpc_status qc_ensure_workspace(ldpc_code c, size_t gamma) {
     DecodeWs &w = c->ws;
-    const size_t need = round_up(gamma, 128);
-    const bool grow = need > w.gamma_cap;
-    const bool stage_missing = want_host_stage && !w.stage_llr;
-    if (!grow && !stage_missing) return LDPC_OK;
-    const size_t cap = grow ? need : w.gamma_cap;
-    if (grow) {
-        // synchronous reallocation (first use or a larger batch)
-        LDPC_CUDA_TRY(cudaDeviceSynchronize());
-        cudaFree(w.msg);
-        cudaFree(w.mu);
-        cudaFree(w.post);
-        cudaFree(w.hw);
-        cudaFree(w.flags);
-        cudaFree(w.iters);
-        cudaFree(w.counters);
-        cudaFree(w.act);
-        cudaFree(w.stage_llr);
-        cudaFree(w.stage_post);
-        cudaFree(w.stage_hard);
-        cudaFree(w.stage_i32);
-        w = DecodeWs();
-        const size_t P32 = cap / 32;
-        if (cudaMalloc(&w.msg, (size_t)c->d.E * cap * 4) != cudaSuccess ||
-            cudaMalloc(&w.mu, (size_t)c->d.N * cap * 4) != cudaSuccess ||
-            cudaMalloc(&w.post, (size_t)c->d.N * cap * 4) != cudaSuccess ||
-            cudaMalloc(&w.hw, (size_t)c->d.N * P32 * 4) != cudaSuccess ||
-            cudaMalloc(&w.flags, P32 * 5 * 4) != cudaSuccess ||
-            cudaMalloc(&w.iters, cap * 2 * 4) != cudaSuccess ||
-            cudaMalloc(&w.counters, 8 * sizeof(unsigned long long)) != cudaSuccess ||
-            cudaMalloc(&w.act, (P32 + 1) * sizeof(int)) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("device allocation for %zu frames failed", cap);
-            return LDPC_ENOMEM;
-        }
-        w.gamma_cap = cap;
-        w.msg_bytes = (size_t)c->d.E * cap * 4;
+    const size_t cap = round_up(gamma, 128);
+    if (cap <= w.gamma_cap) return LDPC_OK;
+    // synchronous reallocation (first use or a larger batch)
+    LDPC_CUDA_TRY(cudaDeviceSynchronize());
+    cudaFree(w.msg);
+    cudaFree(w.mu);
+    cudaFree(w.post);
+    cudaFree(w.hw);
+    cudaFree(w.flags);
+    cudaFree(w.iters);
+    cudaFree(w.counters);
+    cudaFree(w.act);
+    DecodeWs n;
+    n.stage_cap = w.stage_cap;
+    n.stage_llr = w.stage_llr;
+    n.stage_post = w.stage_post;
+    n.stage_hard = w.stage_hard;
+    n.stage_i32 = w.stage_i32;
+    w = n;
+    const size_t P32 = cap / 32;
+    if (cudaMalloc(&w.msg, (size_t)c->d.E * cap * 4) != cudaSuccess ||
+        cudaMalloc(&w.mu, (size_t)c->d.N * cap * 4) != cudaSuccess ||
+        cudaMalloc(&w.post, (size_t)c->d.N * cap * 4) != cudaSuccess ||
+        cudaMalloc(&w.hw, (size_t)c->d.N * P32 * 4) != cudaSuccess ||
+        cudaMalloc(&w.flags, P32 * 5 * 4) != cudaSuccess ||
+        cudaMalloc(&w.iters, cap * 2 * 4) != cudaSuccess ||
+        cudaMalloc(&w.counters, 8 * sizeof(unsigned long long)) != cudaSuccess ||
+        cudaMalloc(&w.act, (P32 + 1) * sizeof(int)) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("device allocation for %zu frames failed", cap);
+        return LDPC_ENOMEM;
     }
-    if (want_host_stage && !w.stage_llr) {
-        if (cudaMalloc(&w.stage_llr, (size_t)c->d.N * cap * 4) != cudaSuccess ||
-            cudaMalloc(&w.stage_post, (size_t)c->d.N * cap * 4) != cudaSuccess ||
-            cudaMalloc(&w.stage_hard, (size_t)c->d.N * cap) != cudaSuccess ||
-            cudaMalloc(&w.stage_i32, cap * 2 * 4) != cudaSuccess) {
-            cudaGetLastError();
-            set_error("device staging allocation for %zu frames failed", cap);
-            return LDPC_ENOMEM;
-        }
+    w.gamma_cap = cap;
+    w.msg_bytes = (size_t)c->d.E * cap * 4;
+    return LDPC_OK;
+}
+
+ldpc_status qc_ensure_stage(ldpc_code c, size_t gamma) {
+    DecodeWs &w = c->ws;
+    const size_t cap = round_up(gamma, 128);
+    if (cap <= w.stage_cap) return LDPC_OK;
+    LDPC_CUDA_TRY(cudaDeviceSynchronize());
+    cudaFree(w.stage_llr);
+    cudaFree(w.stage_post);
+    cudaFree(w.stage_hard);
+    cudaFree(w.stage_i32);
+    w.stage_llr = w.stage_post = nullptr;
+    w.stage_hard = nullptr;
+    w.stage_i32 = nullptr;
+    w.stage_cap = 0;
+    if (cudaMalloc(&w.stage_llr, (size_t)c->d.N * cap * 4) != cudaSuccess ||
+        cudaMalloc(&w.stage_post, (size_t)c->d.N * cap * 4) != cudaSuccess ||
+        cudaMalloc(&w.stage_hard, (size_t)c->d.N * cap) != cudaSuccess ||
+        cudaMalloc(&w.stage_i32, cap * 2 * 4) != cudaSuccess) {
+        cudaGetLastError();
+        set_error("device staging allocation for %zu frames failed", cap);
+        return LDPC_ENOMEM;
     }
+    w.stage_cap = cap;
     return LDPC_OK;
 }
 

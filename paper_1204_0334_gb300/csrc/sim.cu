@@ -459,7 +459,7 @@ ldpc_status qc_ber_sim_refill(ldpc_code c, double sigma, uint64_t seed, uint64_t
     const int V = lanes_per_word(o.msg), W = 32 * V;
     const int P = (gamma + W - 1) / W;
     const size_t slots = (size_t)P * W;
-    ldpc_status st = qc_ensure_workspace(c, slots, 0);
+    ldpc_status st = qc_ensure_workspace(c, slots);
     if (st != LDPC_OK) return st;
     st = sim_ensure(c, c->ws.gamma_cap);
     if (st != LDPC_OK) return st;
