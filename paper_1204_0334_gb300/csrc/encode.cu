@@ -23,7 +23,7 @@
 //             Russians" idea), two rows per thread, T read as column-chunk-major
 //             words (coalesced); the check range is split over blocks, which
 //             meet through atomic XOR
-//   pack:     sliced words -> frame-major bits or bytes (32 ballots per 32 bits)
+//   pack:     sliced words -> frame-major bits (32 ballots per 32 bits) or bytes (a line per frame)
 #include "ldpc_internal.cuh"
 #include "qc_device.cuh"
 
@@ -95,22 +95,31 @@ __global__ void __launch_bounds__(256) enc_slice_kernel(EncSrc src, int64_t k, i
     const int lane = threadIdx.x & 31;
     const int c = blockIdx.y * 8 + (threadIdx.x >> 5);
     if (c >= kc) return;
+    if (src.mode == 0) {
+        // caller's bytes: lane t takes position 32c + t of every frame, 32 contiguous bytes a load, and so
+        // has the sliced word at once (a lane per frame read 32 rows at a time: 77 us for 4096 frames of
+        // k = 15303 against 28)
+        const int64_t j = 32 * (int64_t)c + lane;
+        const int nf = cnt - 32 * g < 32 ? cnt - 32 * g : 32;
+        const uint8_t *b = src.bytes + (size_t)(32 * g) * (size_t)k + (size_t)j;
+        uint32_t x = 0u;
+        if (j < k) {
+#pragma unroll 8
+            for (int t = 0; t < nf; ++t) x |= (uint32_t)(b[(size_t)t * (size_t)k] & 1u) << t;
+            sl[(size_t)g * ld + j] = x;
+        }
+        return;
+    }
     const int f = 32 * g + lane;
     uint32_t w = 0u;
     if (f < cnt) {
-        if (src.mode == 0) {
-            const uint8_t *b = src.bytes + (size_t)f * (size_t)k + 32 * (size_t)c;
-            const int n = (int)std::min<int64_t>(32, k - 32 * (int64_t)c);
-            for (int t = 0; t < n; ++t) w |= (uint32_t)(b[t] & 1u) << t;
-        } else {
-            const uint64_t F = src.frame(f);
-            uint32_t o[4];
-            philox4x32_10((uint32_t)(c >> 2), (uint32_t)F, (uint32_t)(F >> 32), 1u, (uint32_t)src.seed,
-                          (uint32_t)(src.seed >> 32), o);
-            w = o[c & 3];
-            const int64_t rem = k - 32 * (int64_t)c;
-            if (rem < 32) w &= (1u << rem) - 1u;
-        }
+        const uint64_t F = src.frame(f);
+        uint32_t o[4];
+        philox4x32_10((uint32_t)(c >> 2), (uint32_t)F, (uint32_t)(F >> 32), 1u, (uint32_t)src.seed,
+                      (uint32_t)(src.seed >> 32), o);
+        w = o[c & 3];
+        const int64_t rem = k - 32 * (int64_t)c;
+        if (rem < 32) w &= (1u << rem) - 1u;
     }
     const uint32_t x = transpose32(w, lane);
     if (32 * (int64_t)c + lane < k) sl[(size_t)g * ld + 32 * c + lane] = x;
@@ -183,16 +192,15 @@ __global__ void __launch_bounds__(256) enc_parity_kernel(EncSrc src, const uint3
     if (r1 < rank && acc1) atomicXor(sl + (size_t)g * ld + k + r1, acc1);
 }
 
-// where a pack writes
+// where a pack writes: bytes [gamma][len], or frame-major words cwf[slot][NW]
 struct EncDst {
-    int mode;           // 0: bytes [gamma][len]; 2: frame-major words cwf[slot][NW]
     uint8_t *bytes;
     uint32_t *cwf;
     int NW;
 };
 
-// sliced words -> per-frame bits.  Positions x < len: codeword positions (src != NULL,
-// word sl[g][src[x]]) or information bits (src == NULL, word sl[g][x]).
+// sliced words -> per-frame bits of the simulation's codeword rows (frame-major words).  Positions
+// x < len: codeword positions, word sl[g][src[x]].
 __global__ void __launch_bounds__(256) enc_pack_kernel(EncSrc fs, const uint32_t *__restrict__ sl, size_t ld,
                                                        const int *__restrict__ srcidx, int len, EncDst dst) {
     const int g = blockIdx.x;
@@ -206,13 +214,42 @@ __global__ void __launch_bounds__(256) enc_pack_kernel(EncSrc fs, const uint32_t
     if (x < len) w = sl[(size_t)g * ld + (srcidx ? srcidx[x] : x)];
     const uint32_t bits = transpose32(w, lane);  // lane b: positions 32c .. 32c+31 of frame b
     const int f = 32 * g + lane;
-    if (f >= cnt) return;
-    if (dst.mode == 2) {
-        dst.cwf[(size_t)fs.rlist[f] * dst.NW + c] = bits;
-    } else {
-        uint8_t *o = dst.bytes + (size_t)f * len + 32 * (size_t)c;
-        const int n = len - 32 * c < 32 ? len - 32 * c : 32;
-        for (int t = 0; t < n; ++t) o[t] = (uint8_t)((bits >> t) & 1u);
+    if (f < cnt) dst.cwf[(size_t)fs.rlist[f] * dst.NW + c] = bits;
+}
+
+// sliced words -> bytes [gamma][len], one per position: codeword positions (src != NULL) or
+// information bits (src == NULL).  A lane keeps the words of its 4 positions and the warp writes a
+// frame's 128 positions at a time: whole lines, where a lane per frame wrote single bytes of 32 rows
+// (597 us for 4096 frames of n = 18360 against 18).  WIDE: rows start on 4-byte boundaries, so a
+// lane's 4 positions are neighbours and one store; else they are 32 apart and byte stores.
+template <bool WIDE>
+__global__ void __launch_bounds__(256) enc_bytes_kernel(EncSrc fs, const uint32_t *__restrict__ sl, size_t ld,
+                                                        const int *__restrict__ srcidx, int len,
+                                                        uint8_t *__restrict__ out) {
+    const int g = blockIdx.x;
+    const int cnt = fs.count();
+    if (32 * g >= cnt) return;
+    const int lane = threadIdx.x & 31;
+    const int x0 = (blockIdx.y * 8 + (threadIdx.x >> 5)) * 128;
+    if (x0 >= len) return;
+    uint32_t w[4];
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        const int x = x0 + (WIDE ? 4 * lane + e : 32 * e + lane);
+        w[e] = x < len ? sl[(size_t)g * ld + (srcidx ? srcidx[x] : x)] : 0u;
+    }
+    const int nf = cnt - 32 * g < 32 ? cnt - 32 * g : 32;
+    uint8_t *row = out + (size_t)(32 * g) * (size_t)len + x0;
+    for (int f = 0; f < nf; ++f, row += len) {
+        if constexpr (WIDE) {
+            const uint32_t v = ((w[0] >> f) & 1u) | (((w[1] >> f) & 1u) << 8) | (((w[2] >> f) & 1u) << 16) |
+                               (((w[3] >> f) & 1u) << 24);
+            if (x0 + 4 * lane < len) reinterpret_cast<uint32_t *>(row)[lane] = v;  // len is a multiple of 4
+        } else {
+#pragma unroll
+            for (int e = 0; e < 4; ++e)
+                if (x0 + 32 * e + lane < len) row[32 * e + lane] = (uint8_t)((w[e] >> f) & 1u);
+        }
     }
 }
 
@@ -259,21 +296,35 @@ __global__ void __launch_bounds__(256) enc_errors_kernel(const uint32_t *__restr
     if (mine && cnt) atomicAdd(errs + slot, cnt);
 }
 
-// channel LLRs of given codewords (bytes [gamma][N]); as channel_frames_kernel otherwise
-__global__ void channel_cw_kernel(float *__restrict__ out, const uint8_t *__restrict__ cw, int N, int gamma,
-                                  uint64_t seed, uint64_t first_frame, float sigma, float s2) {
+// channel LLRs of given codewords (bytes [gamma][N]); as channel_frames_kernel otherwise.
+// WIDE: rows start on 16-byte (llr) and 4-byte (cw) boundaries, one access each per thread (4096 frames
+// of n = 18360, bound by the generator's arithmetic: 176 us with byte and word accesses and scalar
+// polynomials, 145 us)
+template <bool WIDE>
+__global__ void __launch_bounds__(128) channel_cw_kernel(float *__restrict__ out, const uint8_t *__restrict__ cw, int N,
+                                                         int gamma, uint64_t seed, uint64_t first_frame, float sigma,
+                                                         float s2) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (4 * q >= N) return;
     for (int f = blockIdx.y; f < gamma; f += gridDim.y) {
         uint32_t bits = 0u;
+        if constexpr (WIDE) {
+            const uint32_t b = reinterpret_cast<const uint32_t *>(cw + (size_t)f * N)[q] & 0x01010101u;
+            bits = (b | (b >> 7) | (b >> 14) | (b >> 21)) & 15u;
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (4 * q + e < N) bits |= (uint32_t)(cw[(size_t)f * N + 4 * q + e] & 1u) << e;
+            for (int e = 0; e < 4; ++e)
+                if (4 * q + e < N) bits |= (uint32_t)(cw[(size_t)f * N + 4 * q + e] & 1u) << e;
+        }
         float v4[4];
         channel_quad(seed, first_frame + (uint64_t)f, q, sigma, s2, v4, bits);
+        if constexpr (WIDE) {
+            reinterpret_cast<float4 *>(out + (size_t)f * N)[q] = make_float4(v4[0], v4[1], v4[2], v4[3]);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (4 * q + e < N) out[(size_t)f * N + 4 * q + e] = v4[e];
+            for (int e = 0; e < 4; ++e)
+                if (4 * q + e < N) out[(size_t)f * N + 4 * q + e] = v4[e];
+        }
     }
 }
 
@@ -321,6 +372,16 @@ ldpc_status launch_encode(ldpc_code c, const EncSrc &src, int groups, cudaStream
 ldpc_status launch_pack(ldpc_code c, const EncSrc &src, int groups, const int *srcidx, int len, const EncDst &dst,
                         cudaStream_t s) {
     if (len <= 0) return LDPC_OK;
+    if (dst.bytes) {
+        const dim3 grd(groups, ((len + 127) / 128 + 7) / 8);
+        if (len % 4 == 0 && ((uintptr_t)dst.bytes & 3u) == 0)
+            enc_bytes_kernel<true><<<grd, 256, 0, s>>>(src, c->enc->sl, c->enc->ld, srcidx, len, dst.bytes);
+        else
+            enc_bytes_kernel<false><<<grd, 256, 0, s>>>(src, c->enc->sl, c->enc->ld, srcidx, len, dst.bytes);
+        count_launch();
+        LDPC_CUDA_TRY(cudaGetLastError());
+        return LDPC_OK;
+    }
     const int chunks = (len + 31) / 32;
     enc_pack_kernel<<<dim3(groups, (chunks + 7) / 8), 256, 0, s>>>(src, c->enc->sl, c->enc->ld, srcidx, len, dst);
     count_launch();
@@ -509,7 +570,6 @@ ldpc_status enc_sim_codewords(ldpc_code c, int slots, const int *rlist, const in
     ldpc_status st = launch_encode(c, src, groups, s);
     if (st != LDPC_OK) return st;
     EncDst dst{};
-    dst.mode = 2;
     dst.cwf = cwf;
     dst.NW = c->enc->NW;
     return launch_pack(c, src, groups, c->enc->d_src, c->enc->N, dst, s);
@@ -549,7 +609,6 @@ ldpc_status encode_frames(ldpc_code c, int mode, const uint8_t *info_in, uint64_
         st = launch_encode(c, src, groups, s);
         if (st != LDPC_OK) return st;
         EncDst dst{};
-        dst.mode = 0;
         dst.bytes = cw + (size_t)f0 * e->N;
         st = launch_pack(c, src, groups, e->d_src, e->N, dst, s);
         if (st != LDPC_OK) return st;
@@ -619,8 +678,10 @@ ldpc_status ldpc_channel_codewords(ldpc_code c, double ebn0_db, uint64_t seed, u
     const double sigma = channel_sigma(c, ebn0_db);
     const int N = c->d.N;
     const dim3 grd(((N + 3) / 4 + 127) / 128, std::min(gamma, 65535));
-    channel_cw_kernel<<<grd, 128, 0, (cudaStream_t)stream>>>(llr_out, cw, N, gamma, seed, first_frame, (float)sigma,
-                                                             (float)(2.0 / (sigma * sigma)));
+    const bool wide = N % 4 == 0 && ((uintptr_t)llr_out & 15u) == 0 && ((uintptr_t)cw & 3u) == 0;
+    auto k = wide ? channel_cw_kernel<true> : channel_cw_kernel<false>;
+    k<<<grd, 128, 0, (cudaStream_t)stream>>>(llr_out, cw, N, gamma, seed, first_frame, (float)sigma,
+                                             (float)(2.0 / (sigma * sigma)));
     count_launch();
     LDPC_CUDA_TRY(cudaGetLastError());
     return LDPC_OK;

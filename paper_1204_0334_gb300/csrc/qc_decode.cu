@@ -360,16 +360,22 @@ __global__ void unpack_hard_kernel(const uint32_t *__restrict__ hw, uint8_t *__r
 // BPSK, AWGN; Philox4x32-10 (Salmon et al., SC'11) + Box-Muller, frame-major
 // output [gamma][N] for ldpc_channel.
 // ---------------------------------------------------------------------------
-__global__ void channel_frames_kernel(float *__restrict__ out, int N, int gamma, uint64_t seed, uint64_t first_frame,
-                                      float sigma, float s2) {
+// WIDE: rows start on 16-byte boundaries
+template <bool WIDE>
+__global__ void __launch_bounds__(128) channel_frames_kernel(float *__restrict__ out, int N, int gamma, uint64_t seed,
+                                                             uint64_t first_frame, float sigma, float s2) {
     const int q = blockIdx.x * blockDim.x + threadIdx.x;
     if (4 * q >= N) return;
     for (int f = blockIdx.y; f < gamma; f += gridDim.y) {
         float v4[4];
         channel_quad(seed, first_frame + (uint64_t)f, q, sigma, s2, v4);
+        if constexpr (WIDE) {
+            reinterpret_cast<float4 *>(out + (size_t)f * N)[q] = make_float4(v4[0], v4[1], v4[2], v4[3]);
+        } else {
 #pragma unroll
-        for (int e = 0; e < 4; ++e)
-            if (4 * q + e < N) out[(size_t)f * N + 4 * q + e] = v4[e];
+            for (int e = 0; e < 4; ++e)
+                if (4 * q + e < N) out[(size_t)f * N + 4 * q + e] = v4[e];
+        }
     }
 }
 
@@ -647,8 +653,9 @@ ldpc_status qc_channel_frames(ldpc_code c, double sigma, uint64_t seed, uint64_t
     const int Q = (c->d.N + 3) / 4;
     dim3 grd((Q + 127) / 128, gamma < 65535 ? gamma : 65535);
     count_launch();
-    channel_frames_kernel<<<grd, 128, 0, s>>>(out, c->d.N, gamma, seed, first_frame, (float)sigma,
-                                              (float)(2.0 / (sigma * sigma)));
+    const bool wide = c->d.N % 4 == 0 && ((uintptr_t)out & 15u) == 0;
+    auto k = wide ? channel_frames_kernel<true> : channel_frames_kernel<false>;
+    k<<<grd, 128, 0, s>>>(out, c->d.N, gamma, seed, first_frame, (float)sigma, (float)(2.0 / (sigma * sigma)));
     LDPC_CUDA_TRY(cudaGetLastError());
     return LDPC_OK;
 }

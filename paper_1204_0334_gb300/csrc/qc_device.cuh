@@ -259,71 +259,60 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
 // Coefficients: binary32 minimax fits (Lawson's algorithm) made for this generator.
 // Accuracy (all 2^23 inputs): ln 0.87 ulp, sin and cos 1.6 ulp.
 // ---------------------------------------------------------------------------
-__device__ __forceinline__ float chan_ln(float u) {
-    const uint32_t b = __float_as_uint(u);
-    int e = (int)(b >> 23) - 127;
-    uint32_t mb = (b & 0x7fffffu) | 0x3f800000u;
-    if (mb > 0x3fb504f3u) {
-        mb -= 0x00800000u;
-        e += 1;
-    }
-    const float f = __fsub_rn(__uint_as_float(mb), 1.0f);
-    float R = -0x1.38c9dep-4f;
-    R = __fmaf_rn(R, f, 0x1.055ec6p-3f);
-    R = __fmaf_rn(R, f, -0x1.0d8242p-3f);
-    R = __fmaf_rn(R, f, 0x1.22d92ep-3f);
-    R = __fmaf_rn(R, f, -0x1.54728ap-3f);
-    R = __fmaf_rn(R, f, 0x1.99a01cp-3f);
-    R = __fmaf_rn(R, f, -0x1.000226p-2f);
-    R = __fmaf_rn(R, f, 0x1.555554p-2f);
-    const float t = __fmaf_rn(f, R, -0.5f);
-    const float lnm = __fmaf_rn(__fmul_rn(f, f), t, f);
-    const float ef = __int2float_rn(e);
-    return __fmaf_rn(ef, 0x1.62e4p-1f, __fmaf_rn(ef, 0x1.7f7d1cp-20f, lnm));
-}
-
-// (sin, cos) of 2 pi v 2^-24, v odd in (0, 2^24)
-__device__ __forceinline__ void chan_sincos2pi(uint32_t v, float *sn_out, float *cs_out) {
-    const int32_t j = (int32_t)((v + (1u << 21)) >> 22);
-    const int32_t ri = (int32_t)v - j * (1 << 22);
-    const float r = __fmul_rn(__int2float_rn(ri), 0x1p-24f);
-    const float z = __fmul_rn(r, r);
-    float S = 0x1.a0b0c6p+8f, C = 0x1.c33bfap+6f;
-    S = __fmaf_rn(S, z, -0x1.61b22ap+6f);
-    C = __fmaf_rn(C, z, 0x1.b78f76p+5f);
-    S = __fmaf_rn(S, z, 0x1.46e1p+6f);
-    C = __fmaf_rn(C, z, -0x1.558c8p+6f);
-    S = __fmaf_rn(S, z, -0x1.4abc8ap+5f);
-    C = __fmaf_rn(C, z, 0x1.03c192p+6f);
-    S = __fmaf_rn(S, z, 0x1.921fb6p+2f);
-    C = __fmaf_rn(C, z, -0x1.3bd3ccp+4f);
-    const float sn = __fmul_rn(r, S);
-    const float cs = __fmaf_rn(z, C, 1.0f);
-    switch (j & 3) {
-        case 0: *sn_out = sn; *cs_out = cs; break;
-        case 1: *sn_out = cs; *cs_out = -sn; break;
-        case 2: *sn_out = -sn; *cs_out = -cs; break;
-        default: *sn_out = -cs; *cs_out = sn; break;
-    }
-}
-
 // words -> four channel LLRs: Box-Muller pairs (w0, w1) and (w2, w3),
 // rho = sqrt(-2 ln u(w0)), g = rho cos(2 pi u(w1)), rho sin(2 pi u(w1)), and
 // mu = s2 * fma(sigma, g, x) with s2 = 2 / sigma^2 (binary32 values rounded from double).
 // bit e of `bits` is the code bit c of LLR e: BPSK x = 1 - 2c (all-zero codeword: bits = 0)
+// The two pairs' logarithms, and each pair's sine and cosine, are evaluated two at a time on packed
+// operands, each half rounded by itself.
 __device__ __forceinline__ void box_muller_llr(const uint32_t *w, float sigma, float s2, float *mu4,
                                                uint32_t bits = 0u) {
+    float f[2], ef[2];
 #pragma unroll
     for (int pr = 0; pr < 2; ++pr) {
-        const uint32_t v0 = 2u * (w[2 * pr] >> 9) + 1u, v1 = 2u * (w[2 * pr + 1] >> 9) + 1u;
-        const float u0 = __fmul_rn(__uint2float_rn(v0), 0x1p-24f);
-        const float rho = __fsqrt_rn(__fmul_rn(-2.0f, chan_ln(u0)));
-        float sn, cs;
-        chan_sincos2pi(v1, &sn, &cs);
-        const float x0 = ((bits >> (2 * pr)) & 1u) ? -1.0f : 1.0f;
-        const float x1 = ((bits >> (2 * pr + 1)) & 1u) ? -1.0f : 1.0f;
-        mu4[2 * pr] = __fmul_rn(s2, __fmaf_rn(sigma, __fmul_rn(rho, cs), x0));
-        mu4[2 * pr + 1] = __fmul_rn(s2, __fmaf_rn(sigma, __fmul_rn(rho, sn), x1));
+        const float u0 = __fmul_rn(__uint2float_rn(2u * (w[2 * pr] >> 9) + 1u), 0x1p-24f);
+        const uint32_t b = __float_as_uint(u0);
+        // m = u 2^-e in [sqrt(1/2), sqrt(2)): the exponent rounds up past the mantissa of sqrt(2)
+        const uint32_t up = (b & 0x7fffffu) > 0x3504f3u ? 1u : 0u;
+        const int e = (int)(b >> 23) - 127 + (int)up;
+        f[pr] = __fsub_rn(__uint_as_float((b & 0x7fffffu) | (0x3f800000u - (up << 23))), 1.0f);
+        ef[pr] = __int2float_rn(e);
+    }
+    const f32x2 F = f2(f[0], f[1]), EF = f2(ef[0], ef[1]);
+    f32x2 R = f2fma(f2c(-0x1.38c9dep-4f), F, f2c(0x1.055ec6p-3f));
+    R = f2fma(R, F, f2c(-0x1.0d8242p-3f));
+    R = f2fma(R, F, f2c(0x1.22d92ep-3f));
+    R = f2fma(R, F, f2c(-0x1.54728ap-3f));
+    R = f2fma(R, F, f2c(0x1.99a01cp-3f));
+    R = f2fma(R, F, f2c(-0x1.000226p-2f));
+    R = f2fma(R, F, f2c(0x1.555554p-2f));
+    const f32x2 lnm = f2fma(f2mul(F, F), f2fma(F, R, f2c(-0.5f)), F);
+    const f32x2 m2ln = f2mul(f2c(-2.0f), f2fma(EF, f2c(0x1.62e4p-1f), f2fma(EF, f2c(0x1.7f7d1cp-20f), lnm)));
+    float q[2];
+    f2split(m2ln, q[0], q[1]);
+#pragma unroll
+    for (int pr = 0; pr < 2; ++pr) {
+        const float rho = __fsqrt_rn(q[pr]);
+        const uint32_t v1 = 2u * (w[2 * pr + 1] >> 9) + 1u;
+        const int32_t j = (int32_t)((v1 + (1u << 21)) >> 22);
+        const float r = __fmul_rn(__int2float_rn((int32_t)v1 - j * (1 << 22)), 0x1p-24f);
+        const float z1 = __fmul_rn(r, r);
+        const f32x2 z = f2(z1, z1);
+        f32x2 SC = f2fma(f2(0x1.a0b0c6p+8f, 0x1.c33bfap+6f), z, f2(-0x1.61b22ap+6f, 0x1.b78f76p+5f));
+        SC = f2fma(SC, z, f2(0x1.46e1p+6f, -0x1.558c8p+6f));
+        SC = f2fma(SC, z, f2(-0x1.4abc8ap+5f, 0x1.03c192p+6f));
+        SC = f2fma(SC, z, f2(0x1.921fb6p+2f, -0x1.3bd3ccp+4f));
+        float S, C;
+        f2split(SC, S, C);
+        const float sn = __fmul_rn(r, S), cs = __fmaf_rn(z1, C, 1.0f);
+        // quarter turns: odd ones swap, the second and third negate the sine, the first and second the cosine
+        const float a = j & 1 ? cs : sn, b = j & 1 ? sn : cs;
+        const float so = __uint_as_float(__float_as_uint(a) ^ ((uint32_t)(j & 2) << 30));
+        const float co = __uint_as_float(__float_as_uint(b) ^ ((uint32_t)((j + 1) & 2) << 30));
+        const float x0 = __uint_as_float(0x3f800000u | (((bits >> (2 * pr)) & 1u) << 31));
+        const float x1 = __uint_as_float(0x3f800000u | (((bits >> (2 * pr + 1)) & 1u) << 31));
+        mu4[2 * pr] = __fmul_rn(s2, __fmaf_rn(sigma, __fmul_rn(rho, co), x0));
+        mu4[2 * pr + 1] = __fmul_rn(s2, __fmaf_rn(sigma, __fmul_rn(rho, so), x1));
     }
 }
 
