@@ -32,6 +32,15 @@
 // stop, 4096 frames: 3.17 -> 2.00 ms; 40 frames of the n = 18360 code with early stop: 749 -> 267 us
 // (the launches of all 30 iterations are gone); an irregular n = 2532 code, 1000 frames: 886 -> 377 us.
 //
+// Refill mode (the simulation with a frame-error target that cannot be met, and the streaming decode):
+// every lane of a slot is a frame slot.  A step of a package is three phases: the syndrome, after which
+// frames leave and the next ones enter; the check step with tiles that count wrong bits (or write
+// decision rows) and tiles that draw (or read) the new frames' channel LLRs into the slot's lines; the
+// variable step.  As many slots as L2 holds give the same counts as the caller's number of slots, since
+// a frame's result does not depend on the others.  n = 18360, 32768 frames at 3.5 dB: FP32 68.4 -> 58
+// ms, FP16 59.7 -> 48 ms; the chip computes 78 % of the time (FP32), the rest is the phases' latency at
+// the eight packages that fit.
+//
 // The arithmetic is that of the pass kernels (qc_pipe.cu), operation by operation.
 #include "flow_internal.cuh"
 
@@ -75,7 +84,7 @@ static uint32_t fill_code(const QcDesc &d, int FV, Code &c) {
     // tiles of equal size within a column, in multiples of four variables
     const int vch = (d.p + kc - 1) / kc;
     c.kc = std::min(kc, ((d.p + vch - 1) / vch + 3) / 4 * 4);
-    c.nsyn = (d.M + kComputeWarps * 32 - 1) / (kComputeWarps * 32);
+    c.nsyn = (d.M + kSynRows - 1) / kSynRows;
     c.divp = fast_div((uint32_t)d.p);
     c.rch = fast_div((uint32_t)((d.p + rows - 1) / rows));
     c.rch1 = fast_div((uint32_t)((d.p + rows1 - 1) / rows1));
@@ -89,7 +98,15 @@ static uint32_t fill_code(const QcDesc &d, int FV, Code &c) {
 __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args a) {
     const int *src = reinterpret_cast<const int *>(&st.code);
     int *dst = reinterpret_cast<int *>(a.codes);
-    const int V = st.V;
+    const int V = st.V, kind = a.sim ? F_SYN : F_PACK;
+    if (a.sim) {
+        if (threadIdx.x == 0) *a.sim = st.sim;
+        for (int i = threadIdx.x; i < a.W * 128; i += blockDim.x) {
+            a.simslots[i / 128].age[i % 128] = 0;
+            a.simslots[i / 128].errs[i % 128] = 0;
+            if (i % 128 == 0) a.simslots[i / 128].from = a.simslots[i / 128].to = 0ull;
+        }
+    }
     for (int i = threadIdx.x; i < (int)(sizeof(Code) / 4); i += blockDim.x) dst[i] = src[i];
     if (threadIdx.x == 0) {
         a.ctl->tail = ((unsigned long long)a.W << 40) | ((unsigned long long)a.W * st.tiles);
@@ -100,7 +117,7 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
     for (int n = threadIdx.x; n < kLog; n += blockDim.x) {
         Entry e;
         if (n < a.W) {
-            e.w0 = entry_w0(F_PACK, 0, 1, 0, n);
+            e.w0 = entry_w0(kind, 0, a.sim ? 0 : 1, 0, a.sim ? 0 : n);
             e.w1 = entry_w1((uint32_t)n, n, (uint32_t)(((long long)n * st.tiles) % a.blocks), (uint32_t)st.tiles);
         } else {
             e.w0 = 0ull;
@@ -117,7 +134,7 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
         uint32_t valid = 0u;
         for (int ln = 0; ln < 32; ++ln)
             if ((s * 32 + ln) * V + v < st.code.gamma) valid |= 1u << ln;
-        sl.dn[v] = ~valid;
+        sl.dn[v] = a.sim ? 0xffffffffu : ~valid;  // refill mode: no lane has a frame yet
         sl.un[v] = 0u;
     }
 }
@@ -157,6 +174,18 @@ int flow_slots(const QcDesc &d, int msg, int algo, bool post, int P) {
     return (int)std::min<size_t>({(size_t)P, (size_t)kMaxSlots, std::max<size_t>(fit, 4)});
 }
 
+// Codes of fewer edges fill a tile badly: a phase has few tiles, each with its fixed cost (2500 cycles).
+constexpr int kShortCode = 8000;
+
+// The simulation's frames through flow slots or through launches on all slots (the counts are the
+// same): measured on 4 frames a slot, launches / flow, FP32: 3 x 6, p = 64, 1024 slots 1811 / 1208 us,
+// 4096 slots 2528 / 3571; 4 x 8, p = 118, 4096 slots 5002 / 5779; 4 x 12, p = 211, 4096 slots 7069 /
+// 6013; 4 x 24, p = 765: 68.4 / 59 ms.  FP16 and int8 packages hold two and four times the frames and
+// gain throughout.
+bool flow_sim_pays(const QcDesc &d, int slots, const ldpc_decode_opts &o) {
+    return d.E >= kShortCode || o.msg != LDPC_MSG_F32 || slots <= 2048;
+}
+
 // A phase of the flow takes 6 us however few its tiles (8 with FP16 or int8 messages), a pass of its
 // own launch 4.5 us: with a fixed iteration count the launches are faster below about 80000 message
 // lines (edges times packages).  20 iterations, launches / flow: n = 384, 32 frames (1152 lines) 205 /
@@ -168,49 +197,45 @@ int flow_slots(const QcDesc &d, int msg, int algo, bool post, int P) {
 bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o) {
     const int W = 32 * lanes_per_word(o.msg);
     const long long lines = (long long)d.E * ((gamma + W - 1) / W);
-    const bool shortcode = d.E < 8000;
+    const bool shortcode = d.E < kShortCode;
     return o.early_stop ? !shortcode || lines < 60000 : !shortcode && lines > 80000;
 }
 
-ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int gamma, const ldpc_decode_opts &o,
-                        float *post, uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+// a launch on W slots of m: the code's entry, the buffers, the options
+static ldpc_status prepare(const QcDesc &d, const FlowMem &m, const ldpc_decode_opts &o, int W, bool post, Start &st, Args &a,
+                           uint32_t *tiles) {
     const int V = lanes_per_word(o.msg), FV = o.algo == LDPC_ALGO_MS ? 1 : V;
     if (m.err && *(volatile int *)m.err) {
         set_error("an earlier decode of this object gave up a device-side wait (code %d)", *m.err);
         *m.err = 0;
         return LDPC_ETIMEOUT;
     }
-    Start st;
-    Code &c = st.code;
-    const uint32_t tiles = fill_code(d, FV, c);
-    if (tiles >= (1u << kLogTiles) || gamma / (32 * V) >= (1 << kLogPk) || o.max_iter >= (1 << kLogIt)) {
-        set_error("code too long: %u tiles a phase", tiles);
+    std::memset(&st, 0, sizeof(st));
+    *tiles = fill_code(d, FV, st.code);
+    if (*tiles >= (1u << kLogTiles) || o.max_iter >= (1 << kLogIt)) {
+        set_error("code too long: %u tiles a phase", *tiles);
         return LDPC_EINVAL;
     }
-    c.gamma = gamma;
-    c.llr = llr, c.post = post, c.hard = hard, c.iters = iters, c.ok = ok;
-    c.nparams = o.algo == LDPC_ALGO_NOMS ? o.noms_params : nullptr;
-    Args a;
+    st.code.nparams = o.algo == LDPC_ALGO_NOMS ? o.noms_params : nullptr;
+    st.V = V;
     std::memset(&a, 0, sizeof(a));
     size_t b[4];
-    flow_slot_bytes(d, o.msg, o.algo, post != nullptr, b);
+    flow_slot_bytes(d, o.msg, o.algo, post, b);
     a.slots = (Slot *)m.ctl;
     a.ctl = (Ctl *)((char *)m.ctl + (size_t)m.W * sizeof(Slot));
     a.log = (Entry *)((char *)a.ctl + 256);
     a.codes = (Code *)(a.log + kLog);
     a.ncodes = 1;
-    a.P = (gamma + 32 * V - 1) / (32 * V);
-    a.W = std::min(m.W, a.P);
+    a.W = W;
     a.msg = (uint32_t *)m.msg, a.mu = (uint32_t *)m.mu, a.post = (float *)m.post, a.hw = (uint32_t *)m.hw;
     a.msg_stride = b[0] / 4, a.mu_stride = b[1] / 4, a.post_stride = b[2] / 4, a.hw_stride = b[3] / 4;
-    a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post != nullptr;
+    a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post;
     a.clip = o.clip, a.qscale = ldexpf(1.0f, o.frac_bits), a.lsb = ldexpf(1.0f, -o.frac_bits);
     a.err = m.err;
-    // with several packages in work a phase of its own for the syndrome costs no time and saves the
-    // check step of a package that has stopped; with few it would add its latency to every iteration
-    a.split = a.early && a.W >= 4;
-    st.V = V;
-    st.tiles = (d.N + outv(d.J) - 1) / outv(d.J);
+    return LDPC_OK;
+}
+
+static ldpc_status run(const QcDesc &d, const ldpc_decode_opts &o, Args &a, const Start &st, uint32_t tiles, cudaStream_t s) {
     Shape g{d.J, d.L, 1};
     for (int i = 0; i < d.J * d.L; ++i) g.regular &= d.shift[i] >= 0;
     const int grid = (int)std::min<long long>((long long)tiles * a.W, 1 << 20);
@@ -218,6 +243,26 @@ ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int
     if (o.algo == LDPC_ALGO_NOMS)
         return o.msg == LDPC_MSG_F16 ? run_noms16(a, st, g, grid, s) : run_noms32(a, st, g, grid, s);
     return o.msg == LDPC_MSG_F16 ? run_sp16(a, st, g, grid, s) : run_sp32(a, st, g, grid, s);
+}
+
+ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int gamma, const ldpc_decode_opts &o,
+                        float *post, uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+    const int V = lanes_per_word(o.msg), P = (gamma + 32 * V - 1) / (32 * V);
+    Start st;
+    Args a;
+    uint32_t tiles = 0;
+    const ldpc_status e = prepare(d, m, o, std::min(m.W, P), post != nullptr, st, a, &tiles);
+    if (e != LDPC_OK) return e;
+    Code &c = st.code;
+    c.gamma = gamma;
+    c.llr = llr, c.post = post, c.hard = hard, c.iters = iters, c.ok = ok;
+    a.P = P;
+    // with several long packages in work a phase of its own for the syndrome costs no time and saves the
+    // check step of a package that has stopped; with few, or short ones, it would add its latency to
+    // every iteration (4 x 8, p = 100, 256 frames, FP16: 537 us with, launches 445)
+    a.split = a.early && a.W >= 4 && d.E >= kShortCode;
+    st.tiles = (d.N + outv(d.J) - 1) / outv(d.J);
+    return run(d, o, a, st, tiles, s);
 }
 
 }  // namespace ldpc
@@ -228,8 +273,9 @@ ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int
 struct ldpc_flow_ws {
     size_t cap[4] = {0, 0, 0, 0};
     void *buf[4] = {nullptr, nullptr, nullptr, nullptr};
-    void *ctl = nullptr;
-    int *err = nullptr;  // pinned, device-mapped
+    void *ctl = nullptr, *sim = nullptr;  // sim: the simulation's state and its slots' frames
+    int *err = nullptr;                   // pinned, device-mapped
+    unsigned long long *host = nullptr;   // pinned copy of the simulation's counters
 };
 
 namespace ldpc {
@@ -238,14 +284,14 @@ void flow_free(ldpc_flow_ws *w) {
     if (!w) return;
     for (void *b : w->buf) cudaFree(b);
     cudaFree(w->ctl);
+    cudaFree(w->sim);
+    if (w->host) cudaFreeHost(w->host);
     if (w->err) cudaFreeHost(w->err);
     delete w;
 }
 
-ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
-                             uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
-    const int V = lanes_per_word(o.msg);
-    const int W = flow_slots(c->d, o.msg, o.algo, post != nullptr, (gamma + 32 * V - 1) / (32 * V));
+// buffers for W slots
+static ldpc_status flow_ensure(ldpc_code c, int msg, int algo, bool post, int W, bool sim) {
     auto fail = [&](size_t bytes) {
         cudaGetLastError();
         set_error("device allocation of the decoder's workspace (%zu bytes) failed", bytes);
@@ -267,8 +313,19 @@ ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldp
         }
         *w.err = 0;
     }
+    if (sim && !w.sim) {
+        const size_t need = 512 + kMaxSlots * sizeof(SimSlot);
+        if (cudaMalloc(&w.sim, need) != cudaSuccess) {
+            w.sim = nullptr;
+            return fail(need);
+        }
+    }
+    if (sim && !w.host && cudaHostAlloc((void **)&w.host, 64, cudaHostAllocDefault) != cudaSuccess) {
+        w.host = nullptr;
+        return fail(64);
+    }
     size_t b[4];
-    flow_slot_bytes(c->d, o.msg, o.algo, post != nullptr, b);
+    flow_slot_bytes(c->d, msg, algo, post, b);
     bool synced = false;
     for (int i = 0; i < 4; ++i) {
         const size_t need = b[i] * W;
@@ -284,8 +341,64 @@ ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldp
         }
         w.cap[i] = need;
     }
+    return LDPC_OK;
+}
+
+ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
+                             uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+    const int V = lanes_per_word(o.msg);
+    const int W = flow_slots(c->d, o.msg, o.algo, post != nullptr, (gamma + 32 * V - 1) / (32 * V));
+    const ldpc_status e = flow_ensure(c, o.msg, o.algo, post != nullptr, W, false);
+    if (e != LDPC_OK) return e;
+    const ldpc_flow_ws &w = *c->flow;
     FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.err};
     return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
+}
+
+ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t first_frame, int64_t max_frames, int slots,
+                          const ldpc_decode_opts &o, unsigned long long *h, cudaStream_t s, const StreamIO *io) {
+    const int V = lanes_per_word(o.msg);
+    const int W = flow_slots(c->d, o.msg, o.algo, false, (slots + 32 * V - 1) / (32 * V));
+    ldpc_status e = flow_ensure(c, o.msg, o.algo, false, W, true);
+    if (e != LDPC_OK) return e;
+    ldpc_flow_ws &w = *c->flow;
+    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.err};
+    std::memset(h, 0, 8 * sizeof(*h));
+    constexpr int64_t kMost = (int64_t)1 << 20;  // frames a launch, so that none runs for minutes
+    for (int64_t at = 0; at < max_frames; at += kMost) {
+        Start st;
+        Args a;
+        uint32_t tiles = 0;
+        e = prepare(c->d, m, o, W, false, st, a, &tiles);
+        if (e != LDPC_OK) return e;
+        a.sim = (Sim *)w.sim;
+        a.simslots = (SimSlot *)((char *)w.sim + 512);
+        static_assert(sizeof(Sim) <= 512, "room before the slots");
+        st.tiles = st.code.nsyn;
+        Sim &si = st.sim;
+        si.limit = (unsigned long long)std::min(kMost, max_frames - at);
+        si.first = (io ? 0ull : first_frame) + (unsigned long long)at;
+        si.seed = seed;
+        si.sigma = (float)sigma;
+        si.s2 = (float)(2.0 / (sigma * sigma));
+        if (io) {
+            si.io = 1;
+            si.llr = io->llr, si.hard = io->hard, si.iters = io->iters, si.ok = io->ok;
+            si.wide_in = c->d.N % 4 == 0 && ((uintptr_t)io->llr & 15u) == 0;
+            si.wide_out = c->d.N % 4 == 0 && ((uintptr_t)io->hard & 3u) == 0;
+        }
+        e = run(c->d, o, a, st, tiles, s);
+        if (e != LDPC_OK) return e;
+        LDPC_CUDA_TRY(cudaMemcpyAsync(w.host, a.sim->counters, 64, cudaMemcpyDeviceToHost, s));
+        LDPC_CUDA_TRY(cudaStreamSynchronize(s));
+        if (*(volatile int *)w.err) {
+            set_error("the simulation gave up a device-side wait (code %d)", *w.err);
+            *w.err = 0;
+            return LDPC_ETIMEOUT;
+        }
+        for (int i = 0; i < 8; ++i) h[i] += w.host[i];
+    }
+    return LDPC_OK;
 }
 
 }  // namespace ldpc

@@ -99,7 +99,8 @@ struct Cfg {
     static constexpr int VNW = KC * (JX + FV) * 32;   // words of a variable tile
     static constexpr int STAGE = CNW > VNW ? CNW : VNW;
     static constexpr int OUTV = outv(JX);             // variables of a pack / output tile
-    static constexpr int SYNROWS = kComputeWarps * 32;  // rows of a syndrome tile
+    static constexpr int CHANV = KC * (JX + FV) / FV / 128 * 128;  // variables of a channel tile (whole stage)
+    static constexpr int SYNROWS = kSynRows;
     // pack: OUTV lines of W values with one pad value (bytes for min-sum)
     static_assert((MS ? OUTV * (W + 4) / 4 : OUTV * (W + 1)) <= STAGE, "pack tile");
 };
@@ -116,6 +117,8 @@ struct Smem {
     Desc desc[kStages];
     int dst[kStages][32];       // check tile: the message line of slot l's first row; variable tile: of block row j
     int n1[kStages][32];        // check tile: rows before the wrap of slot l's circulant, -1: absent
+    uint8_t list[kStages][32 * V];  // channel tile: the package's frames that enter, and their ids
+    uint32_t fid[kStages][32 * V];  // (less the launch's first)
     uint32_t hw[kStages][4 * kComputeWarps * V];  // variable tile: the decisions so far (where frames have stopped)
     Code code;                                     // the code of a flow of one code
     alignas(8) unsigned long long full[kStages], used[kStages], empty[kStages];
@@ -163,10 +166,11 @@ __device__ __forceinline__ void phi_pair(float x0, float x1, float &y0, float &y
 // One row of one frame, sum-product: x(l) gives slot l's signed term sign(beta) phi(|beta|) (scaled
 // by SC), out(l, alpha) takes the result.  Prefix sums, then the backward sweep adds the suffix
 // sums (it reads the terms again: twice the shared-memory reads, but 36 registers fewer); phi on
-// pairs of slots.  An infinite term (beta = 0) counts as 1e30, whose sums give the same result
+// pairs of slots.  keep: all ones, or 0 for a frame that has just entered its slot (alpha = 0, so the
+// variable step starts it at beta = mu).  An infinite term (beta = 0) counts as 1e30, whose sums give the same result
 // (phi = 0) and stay finite, so the sweep needs no clamp: that is checked once a row on the whole sum.
 template <int DC, bool REG, int SC, bool FIX, typename X, typename O>
-__device__ __forceinline__ float sp_sweep(uint32_t pm, float clip, X x, O out) {
+__device__ __forceinline__ float sp_sweep(uint32_t pm, float clip, uint32_t keep, X x, O out) {
     float pre[DC / 2];  // the prefix sums before even slots; those before odd ones are one addition away
     uint32_t sgn = 0u;
     float acc = 0.0f;
@@ -196,14 +200,16 @@ __device__ __forceinline__ float sp_sweep(uint32_t pm, float clip, X x, O out) {
         suf += fabsf(t1);
         float m0, m1;
         phi_pair<SC, 1>(a0, a1, m0, m1);
-        out(l, __uint_as_float(__float_as_uint(fminf(m0, clip)) ^ (sgn ^ (__float_as_uint(t0) & 0x80000000u))));
-        out(l - 1, __uint_as_float(__float_as_uint(fminf(m1, clip)) ^ (sgn ^ (__float_as_uint(t1) & 0x80000000u))));
+        const uint32_t s0 = sgn ^ (__float_as_uint(t0) & 0x80000000u), s1 = sgn ^ (__float_as_uint(t1) & 0x80000000u);
+        out(l, __uint_as_float((__float_as_uint(fminf(m0, clip)) ^ s0) & keep));
+        out(l - 1, __uint_as_float((__float_as_uint(fminf(m1, clip)) ^ s1) & keep));
     }
     return 0.0f;
 }
 template <int DC, bool REG, int SC, typename X, typename O>
-__device__ __forceinline__ void sp_row(uint32_t pm, float clip, X x, O out) {
-    if (sp_sweep<DC, REG, SC, false>(pm, clip, x, out) != 0.0f) sp_sweep<DC, REG, SC, true>(pm, clip, x, out);
+__device__ __forceinline__ void sp_row(uint32_t pm, float clip, uint32_t keep, X x, O out) {
+    if (sp_sweep<DC, REG, SC, false>(pm, clip, keep, x, out) != 0.0f)
+        sp_sweep<DC, REG, SC, true>(pm, clip, keep, x, out);
 }
 
 // one row of one frame, normalized/offset min-sum: x(l) gives beta, prm(l) the slot's (w, o)
@@ -233,10 +239,6 @@ __device__ __forceinline__ void noms_row(uint32_t pm, float clip, const float2 *
     }
 }
 
-__device__ __forceinline__ float half_of(uint32_t w, int v) {
-    return __half2float(__ushort_as_half((unsigned short)(v ? w >> 16 : w & 0xffffu)));
-}
-
 // check tile: compute warp `warp` takes rows warp, warp + 8, ... of the tile, in place
 template <typename C, int DC, int V, int RULE, bool REG>
 __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp, int lane, float clip,
@@ -244,6 +246,9 @@ __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp
     constexpr int PITCH = C::ROWS * 32;  // words from one slot's lines to the next slot's
     const uint32_t pm = d.pm;
     if constexpr (RULE == kFlowMS) {
+        uint32_t keep = 0u;  // bytes of the frames that have not just entered
+#pragma unroll
+        for (int v = 0; v < 4; ++v) keep |= ((d.dn[v] >> lane) & 1u) ? 0u : 0xffu << (8 * v);
         for (int r = warp; r < d.rows; r += kComputeWarps) {
             uint32_t *S = stage + r * 32 + lane;
             uint32_t ab[DC], sg[DC];
@@ -267,7 +272,7 @@ __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp
                 const uint32_t eq = __vcmpeq4(ab[l], min1);
                 const uint32_t mag = (min2 & eq) | (min1 & ~eq);
                 const uint32_t sneg = ((sgn ^ sg[l]) >> 7) & 0x01010101u;
-                S[l * PITCH] = __vadd4(mag ^ (sneg * 0xffu), sneg);
+                S[l * PITCH] = __vadd4(mag ^ (sneg * 0xffu), sneg) & keep;
             }
         }
     } else if (d.first && V == 2) {
@@ -291,7 +296,7 @@ __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp
                 noms_row<DC, REG>(pm, clip, prm, [&](int l) { return x[l]; }, put);
             } else {
                 // x + 0 turns -0 into +0 (the sign of a channel LLR is that of x < 0)
-                sp_row<DC, REG, 1>(pm, clip, [&](int l) { return with_sign_of(phi_f(fabsf(x[l])), x[l] + 0.0f); }, put);
+                sp_row<DC, REG, 1>(pm, clip, ~0u, [&](int l) { return with_sign_of(phi_f(fabsf(x[l])), x[l] + 0.0f); }, put);
             }
         }
     } else {
@@ -312,25 +317,20 @@ __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp
                             S[l * PITCH] = __float_as_uint(with_sign_of(phi_f(fabsf(x)), x + 0.0f));
                         }
                     }
-                    sp_row<DC, REG, 1>(pm, clip, [&](int l) { return __uint_as_float(S[l * PITCH]); }, put);
+                    sp_row<DC, REG, 1>(pm, clip, ((d.dn[0] >> lane) & 1u) - 1u,
+                                       [&](int l) { return __uint_as_float(S[l * PITCH]); }, put);
                 }
             } else {
-                uint32_t xw[DC];
-#pragma unroll
-                for (int l = 0; l < DC; ++l) xw[l] = REG || ((pm >> l) & 1u) ? S[l * PITCH] : 0u;
-#pragma unroll
+                // the two frames of a lane word one after the other, each through its half of the words
+                __half *H = reinterpret_cast<__half *>(S);
+#pragma unroll 1
                 for (int v = 0; v < V; ++v) {
+                    auto get = [&](int l) { return __half2float(H[l * PITCH * 2 + v]); };
                     auto put = [&](int l, float a) {
-                        if (REG || ((pm >> l) & 1u)) {
-                            const uint32_t h = __half_as_ushort(__float2half_rn(a));
-                            if (v == 0) xw[l] = (xw[l] & 0xffff0000u) | h;
-                            else S[l * PITCH] = (xw[l] & 0xffffu) | (h << 16);
-                        }
+                        if (REG || ((pm >> l) & 1u)) H[l * PITCH * 2 + v] = __float2half_rn(a);
                     };
-                    if constexpr (RULE == kFlowNOMS)
-                        noms_row<DC, REG>(pm, clip, prm, [&](int l) { return half_of(xw[l], v); }, put);
-                    else
-                        sp_row<DC, REG, 4096>(pm, clip, [&](int l) { return half_of(xw[l], v); }, put);
+                    if constexpr (RULE == kFlowNOMS) noms_row<DC, REG>(pm, clip, prm, get, put);
+                    else sp_row<DC, REG, 4096>(pm, clip, ((d.dn[v] >> lane) & 1u) - 1u, get, put);
                 }
             }
         }
@@ -347,7 +347,7 @@ __device__ __forceinline__ void vn_tile(uint32_t *stage, const uint32_t *hwold, 
     uint32_t frozen[V], any = 0u;
 #pragma unroll
     for (int v = 0; v < V; ++v) frozen[v] = d.dn[v], any |= d.dn[v];
-#pragma unroll 4
+#pragma unroll (V == 1 ? 4 : 1)
     for (int i = warp; i < d.rows; i += kComputeWarps) {
         uint32_t *S = stage + i * 32 + lane;
         uint32_t outb[V];
@@ -476,13 +476,14 @@ __device__ __forceinline__ void pack_tile(uint32_t *stage, const Code &c, const 
     const int f0 = d.pk * W;
     const int nv = min(C::OUTV, c.N - d.n0);
     for (int f = warp; f < W; f += kComputeWarps) {
-        const float *row = c.llr + (size_t)(f0 + f) * c.N + d.n0;
+        // unconditional loads (of the last frame and variable where there is none), so that they overlap
+        const float *row = c.llr + (size_t)min(f0 + f, c.gamma - 1) * c.N + d.n0;
         float x[C::OUTV / 32];
 #pragma unroll
-        for (int q = 0; q < C::OUTV / 32; ++q) {
-            x[q] = MS ? 1e30f : clip;  // frames past the batch
-            if (q * 32 + lane < nv && f0 + f < c.gamma) x[q] = __ldcs(row + q * 32 + lane);
-        }
+        for (int q = 0; q < C::OUTV / 32; ++q) x[q] = __ldcs(row + min(q * 32 + lane, nv - 1));
+        if (f0 + f >= c.gamma)
+#pragma unroll
+            for (int q = 0; q < C::OUTV / 32; ++q) x[q] = MS ? 1e30f : clip;  // frames past the batch
 #pragma unroll
         for (int q = 0; q < C::OUTV / 32; ++q) {
             const int i = q * 32 + lane;
@@ -554,26 +555,31 @@ __device__ __forceinline__ void out_tile(uint32_t *stage, const Code &c, const D
 template <int V>
 __device__ __forceinline__ void syn_tile(const Code &c, const Desc &d, int warp, int lane,
                                          const uint32_t *__restrict__ hw, uint32_t *__restrict__ un) {
+    if (warp >= kSynRows / 32) return;
     const int m = d.n0 + warp * 32 + lane;
     uint32_t syn[V];
 #pragma unroll
     for (int v = 0; v < V; ++v) syn[v] = 0u;
     if (m < c.M) {
         const int j = (int)fdiv((uint32_t)m, c.divp), r = m - j * c.p;
-        for (int l0 = 0; l0 < c.L; l0 += 8) {  // eight edges' loads at a time
-            uint32_t w[8][V];
+        constexpr int B = 24 / V;  // edges whose loads are in flight together
+        for (int l0 = 0; l0 < c.L; l0 += B) {
+            uint32_t w[B][V];
 #pragma unroll
-            for (int i = 0; i < 8; ++i) {
+            for (int i = 0; i < B; ++i) {
+                // absent edges read word 0 and are masked: loads under a condition are not overlapped
+                // (4900 cycles for eight, against 2300)
                 const int l = l0 + i;
                 const int a = l < c.L ? c.sh[j * c.L + l] : -1;
                 int k = r + a;
                 if (k >= c.p) k -= c.p;
-                const uint32_t *h = hw + ((size_t)l * c.p + k) * V;
+                const uint32_t on = a >= 0 ? 0xffffffffu : 0u;
+                const uint32_t *h = hw + (a >= 0 ? ((size_t)l * c.p + k) * V : (size_t)0);
 #pragma unroll
-                for (int v = 0; v < V; ++v) w[i][v] = a >= 0 ? __ldcg(h + v) : 0u;
+                for (int v = 0; v < V; ++v) w[i][v] = __ldcg(h + v) & on;
             }
 #pragma unroll
-            for (int i = 0; i < 8; ++i)
+            for (int i = 0; i < B; ++i)
 #pragma unroll
                 for (int v = 0; v < V; ++v) syn[v] ^= w[i][v];
         }
@@ -582,6 +588,102 @@ __device__ __forceinline__ void syn_tile(const Code &c, const Desc &d, int warp,
     for (int v = 0; v < V; ++v) {
         const uint32_t o = __reduce_or_sync(0xffffffffu, syn[v]);
         if (lane == 0 && o) atomicOr(un + v, o);
+    }
+}
+
+// refill mode: wrong bits (all-zero codeword) of the frames that leave, from their last decisions
+template <int V>
+__device__ __forceinline__ void err_tile(const Code &c, const Desc &d, int warp, int lane,
+                                         const uint32_t *__restrict__ hw, int *__restrict__ errs) {
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const uint32_t ret = d.dn[v];
+        if (!ret) continue;
+        uint32_t w[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int n = d.n0 + warp * 128 + q * 32 + lane;
+            w[q] = n < c.N ? __ldcg(hw + (size_t)n * V + v) & ret : 0u;
+        }
+        int cnt = 0;
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+            for (uint32_t m = __ballot_sync(0xffffffffu, w[q] != 0u); m; m &= m - 1)  // mostly none
+                cnt += (__shfl_sync(0xffffffffu, w[q], __ffs(m) - 1) >> lane) & 1u;
+        if (cnt) atomicAdd(errs + lane * V + v, cnt);
+    }
+}
+
+// streaming: the decisions of the frames that leave, to their rows of the caller's bytes
+template <int V>
+__device__ __forceinline__ void rows_tile(const Code &c, const Sim &si, const SimSlot &ss, const Desc &d, int warp, int lane,
+                                          const uint32_t *__restrict__ hw) {
+    const int n0 = d.n0 + warp * 128;
+    if (n0 >= c.N) return;
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const uint32_t ret = d.dn[v];
+        if (!ret) continue;
+        uint32_t w[4];
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            const int n = n0 + (si.wide_out ? 4 * lane + e : 32 * e + lane);
+            w[e] = n < c.N ? __ldcg(hw + (size_t)n * V + v) : 0u;
+        }
+        for (uint32_t m = ret; m; m &= m - 1) {
+            const int ln = __ffs(m) - 1;
+            uint8_t *row = si.hard + __ldcg(&ss.rfid[ln * V + v]) * (unsigned long long)c.N + n0;
+            if (si.wide_out) {
+                const uint32_t x = ((w[0] >> ln) & 1u) | (((w[1] >> ln) & 1u) << 8) | (((w[2] >> ln) & 1u) << 16) |
+                                   (((w[3] >> ln) & 1u) << 24);
+                if (n0 + 4 * lane < c.N) reinterpret_cast<uint32_t *>(row)[lane] = x;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e)
+                    if (n0 + 32 * e + lane < c.N) row[32 * e + lane] = (uint8_t)((w[e] >> ln) & 1u);
+            }
+        }
+    }
+}
+
+// refill mode: channel LLRs of the frames that enter, into the lines of CHANV variables (in the stage):
+// drawn from the channel, or read from the caller's rows
+template <typename C, int V, bool MS>
+__device__ __forceinline__ void chan_tile(uint32_t *stage, const uint8_t *list, const uint32_t *fid, const Code &c,
+                                          const Sim &si, const Desc &d, int warp, int lane, float clip, float qscale) {
+    constexpr int Q = C::CHANV / 4;
+    const int nf = d.rows, total = nf * Q;
+    // a few frames do not fill the warps: start with another warp in each tile
+    const int first = (warp + d.n0 / C::CHANV * 13) % kComputeWarps;
+    for (int x = first * 32 + lane; x < total; x += kComputeWarps * 32) {
+        // neighbouring lanes: other frames (other banks), or the next quarter-words of the row they read
+        const int i = si.io ? x / Q : x % nf, q = si.io ? x % Q : x / nf;
+        const int f = list[i], n = d.n0 + 4 * q;
+        if (n >= c.N) continue;
+        const unsigned long long F = si.first + fid[i];
+        float y[4];
+        if (si.io) {
+            const float *row = si.llr + F * (unsigned long long)c.N + n;
+            if (si.wide_in) {
+                const float4 t = __ldcs(reinterpret_cast<const float4 *>(row));
+                y[0] = t.x, y[1] = t.y, y[2] = t.z, y[3] = t.w;
+            } else {
+#pragma unroll
+                for (int e = 0; e < 4; ++e) y[e] = n + e < c.N ? __ldcs(row + e) : 0.0f;
+            }
+        } else {
+            channel_quad(si.seed, F, n >> 2, si.sigma, si.s2, y);
+        }
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            if (n + e >= c.N) break;
+            if constexpr (MS) {
+                const float t = fminf(fmaxf(rintf(y[e] * qscale), -127.0f), 127.0f);
+                reinterpret_cast<int8_t *>(stage)[(4 * q + e) * C::W + f] = (int8_t)t;
+            } else {
+                reinterpret_cast<float *>(stage)[(4 * q + e) * C::W + f] = clipf(y[e], clip);
+            }
+        }
     }
 }
 
@@ -661,7 +763,13 @@ __device__ __forceinline__ void open_phase(const Args &a, Slot &sl, int slot, co
                                            int it, int stop) {
     uint32_t tiles = 0;
     switch (kind) {
-        case F_CN: tiles = (a.early && !a.split && it >= 2 ? c.nsyn : 0) + c.J * (it == 1 ? c.rch1.d : c.rch.d); break;
+        case F_CN:
+            if (a.sim) {  // it: bit 0 frames leave, 1 enter, 2 run
+                tiles = (it & 1 ? (c.N + kErrVars - 1) / kErrVars : 0) + (it & 2 ? (c.N + C::CHANV - 1) / C::CHANV : 0) +
+                        (it & 4 ? c.J * c.rch.d : 0);
+                break;
+            }
+            tiles = (a.early && !a.split && it >= 2 ? c.nsyn : 0) + c.J * (it == 1 ? c.rch1.d : c.rch.d); break;
         case F_VN: tiles = c.L * c.vch.d; break;
         case F_FIN:
         case F_SYN: tiles = c.nsyn; break;
@@ -702,16 +810,149 @@ __device__ __forceinline__ void next_package(const Args &a, Slot &sl, int slot) 
     open_phase<C>(a, sl, slot, c, code, pk, F_PACK, 1, stop != 0u);
 }
 
+
 // what finish() needs of a tile
 struct Fin {
     int kind, code, slot, pk, it, stop;
     uint32_t tiles;
 };
 
+// Refill mode, one step of a package complete up to its syndrome (the whole warp): frames whose
+// decisions satisfy every check, or that have run max_iter iterations, leave; the next frames take
+// their lanes.  Returns what the next check phase has to do (bit 0: frames leave, 1: enter, 2: run).
+template <typename C, int V>
+__device__ __forceinline__ int refill(const Args &a, Slot &sl, SimSlot &ss, int lane) {
+    Sim &si = *a.sim;
+    int what = 0;
+    // everything the decision needs in one round of loads
+    uint32_t D[V], U[V];
+    int age[V];
+    unsigned long long id[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        D[v] = __ldcg(&sl.dn[v]), U[v] = __ldcg(&sl.un[v]);
+        age[v] = __ldcg(&ss.age[lane * V + v]);
+        id[v] = __ldcg(&ss.fid[lane * V + v]);
+    }
+    const unsigned long long handed = __ldcg(&si.next);
+    unsigned long long from = __ldcg(&ss.from), to = __ldcg(&ss.to);  // ids the slot has reserved
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const int f = lane * V + v;
+        const bool running = !((D[v] >> lane) & 1u), sat = !((U[v] >> lane) & 1u);
+        const bool ret = running && ((a.early && age[v] >= 1 && sat) || age[v] >= a.max_iter);
+        if (ret) {
+            ss.rfid[f] = id[v];
+            ss.pend[f] = 2 * age[v] + (sat ? 1 : 0);
+            if (si.io) {
+                if (si.iters) si.iters[id[v]] = age[v];
+                if (si.ok) si.ok[id[v]] = sat ? 1 : 0;
+            }
+        }
+        const uint32_t want = __ballot_sync(0xffffffffu, !running || ret);
+        const int need = __popc(want), have = (int)(to - from);
+        unsigned long long more = ~0ull >> 1;
+        int got = 0;
+        if (need > have && handed < si.limit) {
+            // while many frames remain, reserve ahead: one atomic every few steps
+            got = si.limit - handed > 256ull * gridDim.x ? need - have + C::W : need - have;
+            if (lane == 0) more = atomicAdd(&si.next, (unsigned long long)got);
+            more = __shfl_sync(0xffffffffu, more, 0);
+        }
+        const int at = __popc(want & ((1u << lane) - 1u));
+        const unsigned long long idx = at < have ? from + at : more + (unsigned)(at - have);
+        const bool fill = ((want >> lane) & 1u) && idx < si.limit;
+        if (need <= have) from += need;
+        else if (got) from = more + (unsigned)(need - have), to = more + (unsigned)got;
+        else from = to;
+        if (fill) {
+            ss.fid[f] = si.first + idx;
+            ss.age[f] = 0;
+        } else if (running && !ret) {
+            ss.age[f] = age[v] + 1;
+        }
+        const uint32_t retw = __ballot_sync(0xffffffffu, ret), fillw = __ballot_sync(0xffffffffu, fill);
+        const uint32_t dn = (D[v] | retw) & ~fillw;
+        if (lane == 0) {
+            sl.dn[v] = dn;
+            sl.un[v] = 0u;
+            sl.ret[v] = retw;
+            sl.fresh[v] = fillw;
+        }
+        what |= (retw ? 1 : 0) | (fillw ? 2 : 0) | (dn != 0xffffffffu ? 4 : 0);
+    }
+    if (lane == 0) ss.from = from, ss.to = to;
+    // no rows to write and nothing to count: streaming without decisions
+    if (si.io && !si.hard) what &= ~1;
+    return what;
+}
+
+// the frames that left in this step join the totals (the whole warp)
+template <int V>
+__device__ __forceinline__ void tally(const Args &a, Slot &sl, SimSlot &ss, int lane) {
+    unsigned long long t[6] = {0, 0, 0, 0, 0, 0};
+#pragma unroll
+    for (int v = 0; v < V; ++v) {
+        const int f = lane * V + v;
+        if (!((__ldcg(&sl.ret[v]) >> lane) & 1u)) continue;
+        const int pr = __ldcg(&ss.pend[f]), e = __ldcg(&ss.errs[f]);
+        ss.errs[f] = 0;
+        t[0] += 1;
+        t[1] += e > 0;
+        t[2] += (unsigned long long)e;
+        t[3] += (unsigned long long)(pr >> 1);
+        t[4] += e > 0 && (pr & 1);
+        t[5] += (unsigned long long)e * (unsigned long long)e;
+    }
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+        for (int o = 16; o > 0; o >>= 1) t[i] += __shfl_xor_sync(0xffffffffu, t[i], o);
+        if (lane == 0 && t[i]) atomicAdd(&a.sim->counters[i], t[i]);
+    }
+}
+
+// a slot has no frame left (one lane)
+template <typename C>
+__device__ __forceinline__ void end_slot(const Args &a, Slot &sl, int slot) {
+    __threadfence();
+    if (atomicSub(&a.ctl->live, 1) == 1) open_phase<C>(a, sl, slot, a.codes[0], 0, 0, F_EXIT, 0, 0);
+}
+
+// finish() in refill mode: syndrome, check and variable phases in turn
+template <typename C, int V>
+__device__ __forceinline__ void finish_refill(const Args &a, const Code &c, const Fin &d, int lane) {
+    Slot &sl = a.slots[d.slot];
+    SimSlot &ss = a.simslots[d.slot];
+    __syncwarp();
+    uint32_t o = 0u;
+    if (lane == 0) o = add_done(&sl.done, 1u);
+    o = __shfl_sync(0xffffffffu, o, 0);
+    if (o + 1 != d.tiles) return;
+    if (d.kind == F_SYN) {
+        const int what = refill<C, V>(a, sl, ss, lane);
+        __syncwarp();  // opening the phase publishes what the lanes wrote
+        if (lane == 0) {
+            if (what) open_phase<C>(a, sl, d.slot, c, 0, 0, F_CN, what, 0);
+            else end_slot<C>(a, sl, d.slot);
+        }
+    } else if (d.kind == F_VN) {
+        if (lane == 0) open_phase<C>(a, sl, d.slot, c, 0, 0, F_SYN, 0, 0);
+    } else {
+        if ((d.it & 1) && !a.sim->io) tally<V>(a, sl, ss, lane);
+        __syncwarp();
+        if (lane == 0) {
+            if (d.it & 4) open_phase<C>(a, sl, d.slot, c, 0, 0, F_VN, 0, 0);
+            else end_slot<C>(a, sl, d.slot);
+        }
+    }
+    __syncwarp();
+}
+
 // a tile is done: counts it, and opens the slot's next phase with its last one (the whole warp)
 template <typename C, int V>
 __device__ __forceinline__ void finish(const Args &a, const Code &c, const Fin &d, int lane) {
     Slot &sl = a.slots[d.slot];
+    if (a.sim) return finish_refill<C, V>(a, c, d, lane);
     const bool fin = d.it < 0;  // the final syndrome
     if (d.kind == F_SYN) {
         uint32_t o = 0u;
@@ -807,6 +1048,12 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
         if (kind == F_FIN) {
             kind = F_SYN;
             it = -1;
+        } else if (kind == F_CN && a.sim) {
+            const uint32_t ne = it & 1 ? (c.N + kErrVars - 1) / kErrVars : 0;
+            const uint32_t nc = it & 2 ? (c.N + C::CHANV - 1) / C::CHANV : 0;
+            if (idx < ne) kind = a.sim->io ? F_ROWS : F_ERR;
+            else if (idx < ne + nc) kind = F_CHAN, idx -= ne;
+            else idx -= ne + nc;
         } else if (kind == F_CN && a.early && !a.split && it >= 2) {
             if (idx < (uint32_t)c.nsyn) kind = F_SYN;
             else idx -= c.nsyn;
@@ -824,7 +1071,7 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
         const char *msg = reinterpret_cast<const char *>(a.msg + (size_t)slot * a.msg_stride);
         const char *mu = reinterpret_cast<const char *>(a.mu + (size_t)slot * a.mu_stride);
         if (kind == F_CN) {
-            const bool first = it == 1;
+            const bool first = it == 1 && !a.sim;
             const FastDiv &dv = first ? c.rch1 : c.rch;
             const int R = first ? C::ROWS1 : C::ROWS;
             const int j = (int)fdiv(idx, dv), r0 = (int)(idx - (uint32_t)j * dv.d) * R;
@@ -846,6 +1093,8 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
                 d.j = j;
                 d.first = first;
                 d.pm = pm;
+#pragma unroll
+                for (int v = 0; v < V; ++v) d.dn[v] = a.sim ? __ldcg(&a.slots[slot].fresh[v]) : 0u;
                 mbar_arrive_tx(bar, (uint32_t)(__popc(pm) * rows * lb));
             }
             __syncwarp();
@@ -864,7 +1113,7 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
             sm.dst[head][lane] = line;
             uint32_t dn[V];
 #pragma unroll
-            for (int v = 0; v < V; ++v) dn[v] = stop ? __ldcg(&a.slots[slot].dn[v]) : 0u;
+            for (int v = 0; v < V; ++v) dn[v] = stop ? __ldcg(&a.slots[slot].dn[v]) : 0u;  // refill mode: none kept
             if (stop) {  // the decisions of the stopped frames (none yet in the first iteration)
                 const uint32_t *h = a.hw + (size_t)slot * a.hw_stride + (size_t)n0 * V;
                 for (int q = lane; q < K * V; q += 32) sm.hw[head][q] = it > 1 ? __ldcg(h + q) : 0u;
@@ -885,8 +1134,33 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
             if (lane == 31)
                 bulk_load(smem_u32(stage + JX * C::KC * 32), mu + (size_t)n0 * 128 * C::FV,
                           (uint32_t)(K * 128 * C::FV), bar);
+        } else if (kind == F_CHAN) {
+            const int n0 = (int)idx * C::CHANV, K = min(C::CHANV, c.N - n0);
+            int nf = 0;  // the list of the frames that enter
+#pragma unroll
+            for (int v = 0; v < V; ++v) {
+                const uint32_t w = __ldcg(&a.slots[slot].fresh[v]);
+                if ((w >> lane) & 1u) {
+                    const int at = nf + __popc(w & ((1u << lane) - 1u));
+                    sm.list[head][at] = (uint8_t)(lane * V + v);
+                    sm.fid[head][at] = (uint32_t)(__ldcg(&a.simslots[slot].fid[lane * V + v]) - a.sim->first);
+                }
+                nf += __popc(w);
+            }
+            __syncwarp();
+            if (lane == 0) {
+                d.n0 = n0;
+                d.rows = nf;
+                d.j = K;
+                mbar_arrive_tx(bar, (uint32_t)(K * 128 * C::FV));
+                bulk_load(smem_u32(stage), mu + (size_t)n0 * 128 * C::FV, (uint32_t)(K * 128 * C::FV), bar);
+            }
         } else if (lane == 0) {
-            d.n0 = (int)idx * (kind == F_SYN ? C::SYNROWS : C::OUTV);
+            d.n0 = (int)idx * (kind == F_SYN ? C::SYNROWS : (kind == F_ERR || kind == F_ROWS ? kErrVars : C::OUTV));
+            if (kind == F_ERR || kind == F_ROWS) {
+#pragma unroll
+                for (int v = 0; v < V; ++v) d.dn[v] = __ldcg(&a.slots[slot].ret[v]);
+            }
             mbar_arrive(bar);
         }
         __syncwarp();
@@ -923,6 +1197,12 @@ __device__ __forceinline__ void retiring_warp(const Args &a, SM &sm, int st, int
                     bulk_store(msg + line * 128, src, (uint32_t)(rows * 128));
                 }
             }
+            bulk_commit();
+            bulk_wait_read();
+        } else if (kind == F_CHAN) {
+            if (lane == 0)
+                bulk_store(reinterpret_cast<char *>(a.mu + (size_t)d.slot * a.mu_stride) + (size_t)d.n0 * 128 * C::FV,
+                           smem_u32(sm.stage[st]), (uint32_t)(d.j * 128 * C::FV));
             bulk_commit();
             bulk_wait_read();
         }
@@ -984,6 +1264,12 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const Args a) {
             syn_tile<V>(c, d, warp, lane, a.hw + slot * a.hw_stride, a.slots[d.slot].un);
         } else if (kind == F_PACK) {
             pack_tile<C, V, C::MS>(stage, c, d, warp, lane, a.clip, a.qscale, a.mu + slot * a.mu_stride);
+        } else if (kind == F_CHAN) {
+            chan_tile<C, V, C::MS>(stage, sm.list[st], sm.fid[st], c, *a.sim, d, warp, lane, a.clip, a.qscale);
+        } else if (kind == F_ERR) {
+            err_tile<V>(c, d, warp, lane, a.hw + slot * a.hw_stride, a.simslots[slot].errs);
+        } else if (kind == F_ROWS) {
+            rows_tile<V>(c, *a.sim, a.simslots[slot], d, warp, lane, a.hw + slot * a.hw_stride);
         } else if (kind == F_OUT) {
             out_tile<C, V>(stage, c, d, warp, lane, a.hw + slot * a.hw_stride,
                            a.post + slot * a.post_stride);

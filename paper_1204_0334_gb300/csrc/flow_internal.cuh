@@ -24,7 +24,8 @@ __host__ __device__ constexpr int outv(int J) { return J <= 4 ? 256 : 128; }  //
 static_assert(kComputeWarps % 2 == 0, "row, frame pairs of the first iteration");
 
 enum { kFlowSP = 0, kFlowMS = 1, kFlowNOMS = 2 };
-enum { F_PACK = 0, F_CN, F_VN, F_FIN, F_OUT, F_SYN, F_EXIT };  // phases; F_SYN: also a tile of F_CN and F_FIN
+// phases; F_SYN is also a tile of F_CN and F_FIN, the last three are tiles of F_CN in refill mode
+enum { F_PACK = 0, F_CN, F_VN, F_FIN, F_OUT, F_SYN, F_EXIT, F_ERR, F_ROWS, F_CHAN };
 
 // one code of a flow and the caller's buffers of its frames
 struct Code {
@@ -67,6 +68,28 @@ struct alignas(64) Slot {
     unsigned int done, syn_done;  // finished tiles of the open phase, finished syndrome tiles
     int all;                      // every frame has stopped
     uint32_t dn[4], un[4];        // stopped frames, unsatisfied frames (bit = lane)
+    uint32_t ret[4], fresh[4];    // refill mode: frames leaving and entering in this step
+};
+
+// Refill mode (the simulation, and the decode of a large batch by streaming): every package lane is a
+// frame slot that takes the next frame as soon as its frame stops.
+struct Sim {
+    unsigned long long next, limit;  // frames handed out, frames to hand out
+    unsigned long long first;        // id of frame 0
+    unsigned long long counters[8];  // frames, frame errors, bit errors, iterations, undetected, squared bit errors
+    unsigned long long seed;
+    float sigma, s2;
+    const float *llr;                // streaming: the caller's rows, and outputs written as frames leave
+    uint8_t *hard;
+    int32_t *iters, *ok;
+    int io, wide_in, wide_out;       // streaming; rows on 16- / 4-byte boundaries
+};
+struct SimSlot {
+    unsigned long long fid[128], rfid[128];  // frame in the lane, frame that left it in this step
+    int age[128];                            // iterations completed
+    int pend[128];                           // of the frame that left: 2 * iterations + ok
+    int errs[128];                           // its wrong bits
+    unsigned long long from, to;             // frames reserved for the slot
 };
 
 struct Ctl {
@@ -91,6 +114,8 @@ struct Args {
     int blocks;
     float clip, qscale, lsb;
     const int *pkg_code;       // package -> code (NULL: one code)
+    Sim *sim;                  // refill mode, else NULL
+    SimSlot *simslots;
     int *err;                  // host word set when a wait ran out
 };
 
@@ -105,7 +130,8 @@ int resident_blocks(const void *kernel, size_t smem);
 // (start: the launch that opens the first phases, once the number of blocks is known)
 struct Start {
     Code code;
-    int V, tiles;  // lane words' frames; tiles of the pack phase
+    Sim sim;       // refill mode
+    int V, tiles;  // lane words' frames; tiles of the first phase
 };
 ldpc_status run_sp32(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
 ldpc_status run_sp16(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
@@ -113,6 +139,8 @@ ldpc_status run_ms(Args &a, const Start &st, const Shape &g, int tiles, cudaStre
 ldpc_status run_noms32(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
 ldpc_status run_noms16(Args &a, const Start &st, const Shape &g, int tiles, cudaStream_t s);
 ldpc_status start(const Args &a, const Start &st, cudaStream_t s);
+constexpr int kSynRows = 256;                    // rows of a syndrome tile
+constexpr int kErrVars = 128 * kComputeWarps;  // variables of a tile that counts wrong bits or writes decision rows
 
 }  // namespace flow
 
@@ -129,9 +157,14 @@ int flow_slots(const QcDesc &d, int msg, int algo, bool post, int P);
 void flow_slot_bytes(const QcDesc &d, int msg, int algo, bool post, size_t *b4);
 // whether a decode goes to the flow decoder rather than to a launch per pass
 bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o);
+bool flow_sim_pays(const QcDesc &d, int slots, const ldpc_decode_opts &o);
 // Algorithm 1 on gamma frames of a QC code, device buffers in and out (outputs may be NULL)
 ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int gamma, const ldpc_decode_opts &o,
                         float *post, uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
+// refill mode: frames 0 .. max_frames - 1 (ids from first_frame), drawn by the channel or read from io's
+// rows, through min(slots, what stays in L2) frame slots; h: the eight counters.  Waits for the stream.
+ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t first_frame, int64_t max_frames, int slots,
+                          const ldpc_decode_opts &o, unsigned long long *h, cudaStream_t s, const StreamIO *io);
 // the same on a code object, in a workspace that it keeps
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);

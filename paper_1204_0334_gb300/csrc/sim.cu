@@ -34,6 +34,7 @@
 // wrong information bits against their codewords (right after the check, from
 // the decisions the variable pass would otherwise count) and encodes the new
 // frames' codewords before the channel sends them.
+#include "flow_internal.cuh"
 #include "qc_device.cuh"
 
 #include <chrono>
@@ -456,6 +457,10 @@ stream_out_kernel(const uint32_t *__restrict__ hw, const uint32_t *__restrict__ 
 ldpc_status qc_ber_sim_refill(ldpc_code c, double sigma, uint64_t seed, uint64_t first_frame, int64_t max_frames,
                               int64_t target, int gamma, const ldpc_decode_opts &o, unsigned long long *h,
                               cudaStream_t s, const StreamIO *io) {
+    // one launch where the frames' results do not depend on how many are in flight: a frame-error target
+    // that cannot be met (or a caller's batch), all-zero codewords, one rule for every frame
+    if (o.algo != LDPC_ALGO_NOMS && flow_sim_pays(c->d, gamma, o) && (io || (o.codewords == LDPC_CODEWORDS_ZERO && target > max_frames)))
+        return flow_sim_code(c, sigma, seed, first_frame, max_frames, gamma, o, h, s, io);
     const int V = lanes_per_word(o.msg), W = 32 * V;
     const int P = (gamma + W - 1) / W;
     const size_t slots = (size_t)P * W;

@@ -69,3 +69,20 @@ def test_more_packages_than_slots(pkg):
         part = code.decode(mu[f:f + 32], max_iter=12, early_stop=True)
         for a, b in zip(whole, part):
             assert torch.equal(a[f:f + 32], b)
+
+
+@pytest.mark.parametrize("J,L,p,slots,frames", [(3, 6, 17, 32, 1), (3, 6, 64, 128, 700), (4, 12, 31, 4096, 5000),
+                                                (5, 10, 33, 64, 333)])
+@pytest.mark.parametrize("algo,msg", [(0, 0), (1, 2)])
+def test_refill_equals_batch_decode(pkg, J, L, p, slots, frames, algo, msg):
+    """The simulation with a target that cannot be met (one launch, lanes refilled) counts what a batch
+    decode of the same frames counts; fewer frames than lanes, ragged variable counts, several packages."""
+    code = pkg.QCCode(synth.qc_shifts(J, L, p, seed=8), p)
+    r = code.ber_sim(2.0, seed=11, first_frame=5, max_frames=frames, target_frame_errors=1 << 40, gamma=slots,
+                     max_iter=14, early_stop=1, algo=algo, msg=msg)
+    llr = code.channel(2.0, 11, 5, frames)
+    _, hard, it, ok = code.decode(llr, max_iter=14, early_stop=True, algo=algo, msg=msg, want_post=False)
+    e = hard.sum(dim=1).long()
+    assert r["frames"] == frames and r["iters_sum"] == int(it.sum())
+    assert r["bit_errors"] == int(e.sum()) and r["frame_errors"] == int((e > 0).sum())
+    assert r["bit_errors_sq"] == int((e * e).sum()) and r["undetected"] == int(((e > 0) & (ok == 1)).sum())
