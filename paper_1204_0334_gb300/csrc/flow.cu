@@ -16,9 +16,10 @@
 //    (handing tiles out by atomics: 3200 cycles a tile in the block's serial part).  With several
 //    packages in work the chip stays full through phase ends, and a package stops the moment its
 //    frames have.
-//  * No tile waits for another: a block that has a tile always finishes it, so any number of resident
-//    blocks makes progress on the tiles that are theirs; all of a launch's blocks are resident (one an
-//    SM).  Every wait has a limit, after which the launch ends and the object reports a timeout.
+//  * No tile waits for another, but a phase ends with the last of its tiles, whichever block it fell
+//    to: the launch is cooperative, so its blocks (one an SM) are all resident even where another
+//    stream's kernel holds SMs.  Every wait has a limit, after which the launch ends and the object
+//    reports a timeout.
 //  * Within a block, one warp reads the log and starts the bulk copies of its tiles' lines (the rows
 //    of a tile meet each circulant in one run of consecutive edges, or two at its wrap: a copy and an
 //    address per slot of all the tile's rows, not per edge); 24 warps compute out of shared memory and

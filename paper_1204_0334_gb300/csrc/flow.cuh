@@ -1297,7 +1297,18 @@ static ldpc_status launch(Args &a, const Start &st, int tiles, cudaStream_t s) {
     a.blocks = std::min({tiles, most, 1 << kLogBase});
     const ldpc_status e = start(a, st, s);
     if (e != LDPC_OK) return e;
-    k<<<a.blocks, kThreads, smem, s>>>(a);
+    // cooperative: all blocks resident or none, whatever else runs on the device
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at[1];
+    cfg.gridDim = dim3((unsigned)a.blocks);
+    cfg.blockDim = dim3(kThreads);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at[0].id = cudaLaunchAttributeCooperative;
+    at[0].val.cooperative = 1;
+    cfg.attrs = at;
+    cfg.numAttrs = 1;
+    LDPC_CUDA_TRY(cudaLaunchKernelEx(&cfg, k, a));
     count_launch();
     LDPC_CUDA_TRY(cudaGetLastError());
     return LDPC_OK;
