@@ -391,10 +391,15 @@ ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc
     uint8_t *d_hard = hard && pointer_kind(hard) == 1 ? w.stage_hard : hard;
     int32_t *d_iters = iters && pointer_kind(iters) == 1 ? w.stage_i32 : iters;
     int32_t *d_ok = ok && pointer_kind(ok) == 1 ? w.stage_i32 + w.stage_cap : ok;
-    if (!c->sparse && flow_pays(c->d, gamma, o)) {
+    bool on_chip = false;
+    if (!c->sparse) {
+        st = chip_decode(c->d, src, gamma, o, d_post, d_hard, d_iters, d_ok, s, &on_chip);
+        if (st != LDPC_OK) return st;
+    }
+    if (!on_chip && !c->sparse && flow_pays(c->d, gamma, o)) {
         st = flow_decode_code(c, src, gamma, o, d_post, d_hard, d_iters, d_ok, s);
         if (st != LDPC_OK) return st;
-    } else {
+    } else if (!on_chip) {
         st = qc_ensure_workspace(c, (size_t)gamma);
         if (st != LDPC_OK) return st;
         st = qc_pack_llr(c, src, gamma, o, s);

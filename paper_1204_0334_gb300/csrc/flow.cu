@@ -194,11 +194,13 @@ bool flow_sim_pays(const QcDesc &d, int slots, const ldpc_decode_opts &o) {
 // 128 frames (115200) 465 / 394.  Short codes fill a tile badly: 3 x 6, p = 64, 2048 frames (73728)
 // 419 / 572, 4 x 8, p = 100, 2048 frames (204800) 720 / 801.  With early stop the flow ends with the
 // last frame and its syndrome takes no launches, so it is taken unless the code is short and the
-// batch large.
+// batch large.  FP32 packages hold the fewest frames, so a large batch has the most phases, and a code
+// counts as short there up to 10000 edges (4 x 24, p = 100: 512 frames 557 / 490, 2048 frames 1592 /
+// 1735, with early stop 1591 / 1867; 4 x 12, p = 211: 1994 / 1695).
 bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o) {
     const int W = 32 * lanes_per_word(o.msg);
     const long long lines = (long long)d.E * ((gamma + W - 1) / W);
-    const bool shortcode = d.E < kShortCode;
+    const bool shortcode = d.E < kShortCode || (o.msg == LDPC_MSG_F32 && d.E < 10000 && lines > 400000);
     return o.early_stop ? !shortcode || lines < 60000 : !shortcode && lines > 80000;
 }
 

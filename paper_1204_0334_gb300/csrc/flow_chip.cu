@@ -1,0 +1,116 @@
+// The on-chip decoder: Algorithm 1 on a few packages of a short code, one launch, a thread-block
+// cluster per package.
+//
+// A short code's pass takes a launch 4.5 us, and a phase of the flow decoder 6, for a few hundred
+// nanoseconds of work.  Here the blocks of a cluster divide a package's variables and keep everything of
+// theirs in shared memory: channel LLRs, messages (by variable, as in global memory), decision words,
+// posteriors.  The variable step is local; the check step reads and writes its edges in the other
+// blocks' shared memory; two hardware cluster barriers an iteration, and no spinning.  Early stop ends
+// the launch with the package's last frame: the syndrome goes with the check step, a warp per row, a
+// lane per edge.
+//
+// The blocks of a cluster are as many as leave all packages resident at once (16, 8, 4, 2 or 1): more
+// blocks a package, fewer rows a warp.  What bounds it is latency: the chain of a row (its remote loads
+// in flight together, then the sums and transforms) and the barriers.  n = 384, 32 frames, 30 iterations:
+// 283 us by launches, 86 here
+// (3500 cycles an iteration in the check step and its barrier, 2300 in the variable step and its own).
+//
+// The arithmetic is that of the pass kernels (qc_pipe.cu), operation by operation.
+#include "flow_internal.cuh"
+
+#include <algorithm>
+#include <cmath>
+#include <cstring>
+#include <map>
+#include <mutex>
+#include <utility>
+
+namespace ldpc {
+namespace chip {
+
+using namespace flow;
+
+size_t bytes(const Code &c, int V, bool ms, bool post, int NC) {
+    const size_t W = 32 * V;
+    return (size_t)NC * 4 * ((size_t)c.J * 32 + (ms ? 33 : W + 1) + V + (post ? W + 1 : 0));
+}
+
+// Message lines of a block beyond which the passes over the whole chip are faster: an SM works through
+// its lines of an iteration one after another.  20 iterations, the faster of launches and flow / here, us,
+// at lines a block: FP32 633: 290 / 263 (1 package), 329 / 267 (4); 800: 462 / 284 (32).  FP16 320: 293 /
+// 307 (1), with early stop 451 / 342; 400: 372 / 292 (8); 633: 290 / 471 (1), 372 / 479 (2); 800: 461 / 491
+// (16), 648 / 507 (32).  int8 400: 336 / 226 (8); 600: 299 / 342 (1), 388 / 350 (4); 640: 426 / 349 (8).
+static int most_lines(int V, int P, bool early) {
+    if (V == 1) return 800;
+    if (V == 2) return P < 4 && !early ? 300 : P < 24 ? 400 : 800;
+    return P < 4 ? 500 : 800;
+}
+
+int pick(const void *kernel, const Code &c, int V, bool ms, const ChipArgs &a, int P) {
+    static std::mutex mu;
+    static std::map<std::pair<const void *, int>, int> active;  // clusters resident at once, one block an SM
+    std::lock_guard<std::mutex> lk(mu);
+    int E = 0;
+    for (int i = 0; i < c.J * c.L; ++i) E += c.sh[i] >= 0 ? c.p : 0;
+    for (int C = 16; C >= 1; C /= 2) {
+        const int NC = (c.N + C - 1) / C;
+        if (bytes(c, V, ms, a.want_post, NC) > kChipMost || E > C * most_lines(V, P, a.early)) return 0;  // fewer blocks hold less
+        if ((C - 1) * NC >= c.N) continue;  // a block would have no variable
+        const auto key = std::make_pair(kernel, C);
+        auto f = active.find(key);
+        if (f == active.end()) {
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChipMost);
+            cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+            cudaLaunchConfig_t cfg{};
+            cudaLaunchAttribute at[1];
+            cfg.gridDim = dim3((unsigned)C);
+            cfg.blockDim = dim3(kChipThreads);
+            cfg.dynamicSmemBytes = kChipMost;
+            at[0].id = cudaLaunchAttributeClusterDimension;
+            at[0].val.clusterDim.x = C;
+            at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+            cfg.attrs = at;
+            cfg.numAttrs = 1;
+            int n = 0;
+            if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
+                cudaGetLastError();
+                n = 0;
+            }
+            f = active.emplace(key, n).first;
+        }
+        if (P <= f->second) return C;
+    }
+    return 0;
+}
+
+}  // namespace chip
+
+using namespace flow;
+
+// Takes a decode whose packages all fit on the chip at once; *taken says whether it did.
+ldpc_status chip_decode(const QcDesc &d, const float *llr, int gamma, const ldpc_decode_opts &o, float *post, uint8_t *hard,
+                        int32_t *iters, int32_t *ok, cudaStream_t s, bool *taken) {
+    const int V = lanes_per_word(o.msg), P = (gamma + 32 * V - 1) / (32 * V);
+    *taken = false;
+    if (P > 152 || d.E > 16 * 800) return LDPC_OK;
+    Code c;
+    std::memset(&c, 0, sizeof(c));
+    c.J = d.J, c.L = d.L, c.p = d.p, c.N = d.N, c.M = d.M;
+    c.divp = d.divP;
+    std::memcpy(c.sh, d.shift, sizeof(int) * d.J * d.L);
+    c.gamma = gamma;
+    c.llr = llr, c.post = post, c.hard = hard, c.iters = iters, c.ok = ok;
+    c.nparams = o.algo == LDPC_ALGO_NOMS ? o.noms_params : nullptr;
+    chip::ChipArgs a;
+    std::memset(&a, 0, sizeof(a));
+    a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post != nullptr;
+    a.clip = o.clip, a.qscale = ldexpf(1.0f, o.frac_bits), a.lsb = ldexpf(1.0f, -o.frac_bits);
+    if (o.algo == LDPC_ALGO_MS) return chip::run_ms(c, a, P, s, taken);
+    if (o.algo == LDPC_ALGO_NOMS)
+        return o.msg == LDPC_MSG_F16 ? chip::run_noms16(c, a, P, s, taken)
+                                     : chip::run_noms32(c, a, P, s, taken);
+    return o.msg == LDPC_MSG_F16 ? chip::run_sp16(c, a, P, s, taken)
+                                 : chip::run_sp32(c, a, P, s, taken);
+}
+
+}  // namespace ldpc

@@ -169,4 +169,31 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
 
+// the on-chip decoder of short codes (flow_chip.cu)
+ldpc_status chip_decode(const QcDesc &d, const float *llr, int gamma, const ldpc_decode_opts &o, float *post, uint8_t *hard,
+                        int32_t *iters, int32_t *ok, cudaStream_t s, bool *taken);
+
+namespace chip {
+
+constexpr int kChipThreads = 512;
+constexpr size_t kChipMost = 225 * 1024;  // with the static arrays, below the 227 KB a block may have
+// one block an SM, also where registers and shared memory would let two in
+constexpr size_t kChipLeast = 116 * 1024;
+
+struct ChipArgs {
+    int C, NC;       // blocks of a cluster, variables of a block
+    FastDiv divNC;
+    int max_iter, early, want_post;
+    float clip, qscale, lsb;
+};
+size_t bytes(const flow::Code &c, int V, bool ms, bool post, int NC);
+// blocks of a cluster so that all P packages are resident, or 0
+int pick(const void *kernel, const flow::Code &c, int V, bool ms, const ChipArgs &a, int P);
+ldpc_status run_sp32(const flow::Code &c, ChipArgs &a, int P, cudaStream_t s, bool *taken);
+ldpc_status run_sp16(const flow::Code &c, ChipArgs &a, int P, cudaStream_t s, bool *taken);
+ldpc_status run_ms(const flow::Code &c, ChipArgs &a, int P, cudaStream_t s, bool *taken);
+ldpc_status run_noms32(const flow::Code &c, ChipArgs &a, int P, cudaStream_t s, bool *taken);
+ldpc_status run_noms16(const flow::Code &c, ChipArgs &a, int P, cudaStream_t s, bool *taken);
+
+}  // namespace chip
 }  // namespace ldpc

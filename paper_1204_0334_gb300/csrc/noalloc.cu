@@ -127,6 +127,11 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
     noalloc_need(c->d, cap, off);
     unsigned char *base = (unsigned char *)base_v;
     cudaStream_t s = (cudaStream_t)stream;
+    if (!c->sparse) {
+        bool on_chip = false;
+        st = chip_decode(c->d, llr, gamma, o, post, hard, iters, ok, s, &on_chip);
+        if (st != LDPC_OK || on_chip) return st;
+    }
     if (!c->sparse && flow_pays(c->d, gamma, o)) {
         // the slots' buffers one after another: a slot takes no more than its package's share of the
         // bytes counted above (the decision words' rounding fits in the iteration counts', not kept here)
