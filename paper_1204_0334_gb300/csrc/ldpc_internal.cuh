@@ -155,9 +155,6 @@ ldpc_status qc_vn_pipe(ldpc_code c, const ldpc_decode_opts &o, bool stop, bool p
 // packages with a running frame
 ldpc_status qc_compact(ldpc_code c, int P, int V, cudaStream_t s);
 // general (index-table) codes (qc_pipe.cu, sparse.cu)
-ldpc_status qc_cn_pipe_sparse(ldpc_code c, const ldpc_decode_opts &o, cudaStream_t s);
-ldpc_status qc_vn_pipe_sparse(ldpc_code c, const ldpc_decode_opts &o, bool stop, bool post, int it, int par,
-                              cudaStream_t s);
 ldpc_status sparse_decode_device(ldpc_code c, int gamma, const ldpc_decode_opts &o, bool want_post, cudaStream_t s);
 ldpc_status qc_init_flags(ldpc_code c, int gamma, int V, cudaStream_t s);
 ldpc_status qc_finish_frames(ldpc_code c, int gamma, const ldpc_decode_opts &o, cudaStream_t s);

@@ -340,6 +340,17 @@ __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;\n" ::"n"(N) : "memory");
 }
 
+// a word that is loaded only where `on` (a predicated load: loads in a row overlap, which the compiler does
+// not arrange for loads under a branch), else 0
+__device__ __forceinline__ uint32_t load_if(const uint32_t *p, bool on) {
+    uint32_t x = 0u;
+    asm volatile("{\n .reg .pred q;\n setp.ne.u32 q, %2, 0;\n @q ld.global.u32 %0, [%1];\n}"
+                 : "+r"(x)
+                 : "l"(p), "r"((uint32_t)on)
+                 : "memory");
+    return x;
+}
+
 // blocks of a persistent launch: resident blocks per SM (occupancy API, cached per
 // kernel and dynamic shared-memory size) times the SM count; also raises the kernel's
 // dynamic shared-memory limit to the largest size requested so far
