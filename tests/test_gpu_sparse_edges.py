@@ -1,11 +1,11 @@
 """General codes whose columns have every degree from 1 to 8 and rows every kernel width up to 32, with
-ragged variable and frame counts."""
+ragged variable and frame counts; and convolutional codes with an odd number of variables a frame."""
 import numpy as np
 import pytest
 
 import oracle
 import synth
-from test_gpu_ldpccc import pkg  # noqa: F401  (the module's fixture)
+from test_gpu_ldpccc import compare, pkg, run_gpu  # noqa: F401  (the module's fixture)
 
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
@@ -34,3 +34,13 @@ def test_every_degree(pkg, N, M, gamma, early):
         assert run.any()
         err = np.abs(post.cpu().numpy() - po) / np.maximum(1.0, np.abs(po))
         assert np.max(err[run]) <= tol, msg
+
+
+@pytest.mark.parametrize("J,L,p", [(3, 9, 7), (1, 5, 11)])
+def test_ldpccc_odd_frames(pkg, J, L, p):
+    shifts = synth.qc_shifts(J, L, p, seed=3)
+    c = pkg.LDPCCC(shifts, p, 3, 40).c
+    assert c % 2 == 1
+    mu = synth.gaussian_llrs(40, 14 * c, seed=2, ebn0_db=2.0, rate=0.5).reshape(40, 14, c)
+    hard, post, decided = run_gpu(pkg, shifts, p, 3, mu, [5, 9])
+    compare(shifts, p, 3, mu, hard, post, decided, f"odd frames {J}x{L}")
