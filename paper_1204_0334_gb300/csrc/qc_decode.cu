@@ -577,7 +577,8 @@ ldpc_status qc_decode_device(ldpc_code c, int gamma, const ldpc_decode_opts &o, 
         }
         prof_end(slot_cn, s);
         const int slot_vn = prof_begin(1, s);
-        st = qc_vn_pipe(c, o, syn, want_post, it, par, s);
+        // without early stop only the last iteration's posteriors are read
+        st = qc_vn_pipe(c, o, syn, want_post && (o.early_stop || it == o.max_iter), it, par, s);
         if (st != LDPC_OK) return st;
         prof_end(slot_vn, s);
         count_launch(2);
