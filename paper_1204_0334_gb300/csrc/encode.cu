@@ -104,8 +104,20 @@ __global__ void __launch_bounds__(256) enc_slice_kernel(EncSrc src, int64_t k, i
         const uint8_t *b = src.bytes + (size_t)(32 * g) * (size_t)k + (size_t)j;
         uint32_t x = 0u;
         if (j < k) {
+            if (nf == 32) {
 #pragma unroll 8
-            for (int t = 0; t < nf; ++t) x |= (uint32_t)(b[(size_t)t * (size_t)k] & 1u) << t;
+                for (int t = 0; t < 32; ++t) x |= (uint32_t)(b[(size_t)t * (size_t)k] & 1u) << t;
+            } else {
+                // a last, partial group: eight loads in flight as well (the last frame's again past the end)
+                for (int t0 = 0; t0 < nf; t0 += 8) {
+                    uint8_t v[8];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) v[t] = b[(size_t)(t0 + t < nf ? t0 + t : nf - 1) * (size_t)k];
+#pragma unroll
+                    for (int t = 0; t < 8; ++t) x |= (uint32_t)(v[t] & 1u) << (t0 + t);
+                }
+                x &= (1u << nf) - 1u;
+            }
             sl[(size_t)g * ld + j] = x;
         }
         return;
@@ -232,12 +244,17 @@ __global__ void __launch_bounds__(256) enc_bytes_kernel(EncSrc fs, const uint32_
     const int lane = threadIdx.x & 31;
     const int x0 = (blockIdx.y * 8 + (threadIdx.x >> 5)) * 128;
     if (x0 >= len) return;
+    // the four loads in flight together: positions past the end read the last one and are not stored
+    int at[4];
     uint32_t w[4];
 #pragma unroll
-    for (int e = 0; e < 4; ++e) {
-        const int x = x0 + (WIDE ? 4 * lane + e : 32 * e + lane);
-        w[e] = x < len ? sl[(size_t)g * ld + (srcidx ? srcidx[x] : x)] : 0u;
+    for (int e = 0; e < 4; ++e) at[e] = min(x0 + (WIDE ? 4 * lane + e : 32 * e + lane), len - 1);
+    if (srcidx) {
+#pragma unroll
+        for (int e = 0; e < 4; ++e) at[e] = srcidx[at[e]];
     }
+#pragma unroll
+    for (int e = 0; e < 4; ++e) w[e] = sl[(size_t)g * ld + at[e]];
     const int nf = cnt - 32 * g < 32 ? cnt - 32 * g : 32;
     uint8_t *row = out + (size_t)(32 * g) * (size_t)len + x0;
     for (int f = 0; f < nf; ++f, row += len) {
