@@ -126,13 +126,16 @@ ldpc_status ldpc_code_dims(ldpc_code code, int64_t *N, int64_t *M, int64_t *E, i
  * Streaming: for a QC code with opts->early_stop, sum-product with F32 messages
  * or integer min-sum, post == NULL, gamma at least twice the slot count (the
  * one ldpc_tune_slots picked for this code and algo/msg, else 4096) and every
- * buffer in device or pinned host memory, the frames stream through that many
+ * buffer in device or pinned host memory, the frames stream through frame
  * slots as in ldpc_ber_sim: a frame enters a slot as soon as the previous one
  * stops, reading its LLR row directly (pinned host rows through their device
  * mapping, no staging copy), and writes its decisions, iteration count and ok
  * flag when it stops.  Each frame gets exactly the iterations and decisions of
  * the batch path.  This form returns when the batch is decoded (it synchronizes
  * the stream).
+ * A batch of a QC code runs as one launch where that is faster; every form gives
+ * the same results.  If a wait on the device gives up (it has a limit), a form that
+ * does not synchronize reports LDPC_ETIMEOUT on the next call on the code.
  * Errors: LDPC_EINVAL (null code/llr, gamma < 1, bad opts), LDPC_EUNSUPPORTED
  * (algo/msg pair not built), LDPC_ENOMEM, LDPC_ECUDA, LDPC_ETIMEOUT.
  */
@@ -283,7 +286,8 @@ typedef struct {
  * draw them, errors counted over the information bits), so a run can be
  * resumed from (seed, first_frame + out->frames) and partial results added.
  * Blocks the calling thread until the run ends (it reads the totals every
- * two steps).
+ * two steps, or at the end of a run whose error target is above max_frames;
+ * such a run may keep fewer frames in flight than gamma, with the same counts).
  *   gamma: frame slots; 0 = the slot count ldpc_tune_slots picked for this code and
  *   opts->algo / opts->msg (tuned on the spot, at this Eb/N0 and seed, if it has not been).
  *   out: host pointer, filled on return.

@@ -577,7 +577,9 @@ ldpc_status qc_decode_device(ldpc_code c, int gamma, const ldpc_decode_opts &o, 
         }
         prof_end(slot_cn, s);
         const int slot_vn = prof_begin(1, s);
-        // without early stop only the last iteration's posteriors are read
+        // without early stop only the last iteration's posteriors are read (20 iterations, written by all /
+        // by the last: 4 x 24, p = 100, 2048 frames, FP32 1603 / 1540 us; 4 x 16, p = 80, 512 frames, FP16
+        // 469 / 429)
         st = qc_vn_pipe(c, o, syn, want_post && (o.early_stop || it == o.max_iter), it, par, s);
         if (st != LDPC_OK) return st;
         prof_end(slot_vn, s);

@@ -1,6 +1,10 @@
 // Continuous Monte-Carlo simulation (the protocol of Sec. V) with frame slots
 // that are refilled as soon as their frame stops.
 //
+// This file's launches serve runs with an error target that can be met, random codewords, the learned
+// min-sum and short FP32 codes on many slots; the other runs go to the flow decoder's refill mode
+// (flow.cu) and count the same.
+//
 // Decoding gamma frames to the end before drawing the next gamma wastes most of
 // the early-stopping gain: a package of 32 frames keeps being visited until its
 // slowest frame stops, and the whole batch waits for the slowest package.
