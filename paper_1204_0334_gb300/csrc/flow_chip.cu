@@ -37,12 +37,13 @@ size_t bytes(const Code &c, int V, bool ms, bool post, int NC) {
 
 // Message lines of a block beyond which the passes over the whole chip are faster: an SM works through
 // its lines of an iteration one after another.  20 iterations, the faster of launches and flow / here, us,
-// at lines a block: FP32 633: 290 / 263 (1 package), 329 / 267 (4); 800: 462 / 284 (32).  FP16 320: 293 /
-// 307 (1), with early stop 451 / 342; 400: 372 / 292 (8); 633: 290 / 471 (1), 372 / 479 (2); 800: 461 / 491
-// (16), 648 / 507 (32).  int8 400: 336 / 226 (8); 600: 299 / 342 (1), 388 / 350 (4); 640: 426 / 349 (8).
-static int most_lines(int V, int P, bool early) {
+// at lines a block (and packages): FP32 633: 290 / 263 (1), 329 / 267 (4); 800: 462 / 284 (32).  FP16 320: 298
+// / 256 (1); 390: 334 / 264 (2); 400: 372 / 254 (8); 800: 461 / 491 (16), 648 / 507 (32); rows of more than 16
+// slots, which take a frame of a word after the other, 375: 341 / 427 (1), with early stop 462 / 450.  int8
+// 400: 336 / 226 (8); 600: 299 / 342 (1), 388 / 350 (4); 640: 426 / 349 (8).
+static int most_lines(const Code &c, int V, int P, bool early) {
     if (V == 1) return 800;
-    if (V == 2) return P < 4 && !early ? 300 : P < 24 ? 400 : 800;
+    if (V == 2) return P >= 24 ? 800 : c.L > 16 && !early ? 250 : 400;
     return P < 4 ? 500 : 800;
 }
 
@@ -54,7 +55,7 @@ int pick(const void *kernel, const Code &c, int V, bool ms, const ChipArgs &a, i
     for (int i = 0; i < c.J * c.L; ++i) E += c.sh[i] >= 0 ? c.p : 0;
     for (int C = 16; C >= 1; C /= 2) {
         const int NC = (c.N + C - 1) / C;
-        if (bytes(c, V, ms, a.want_post, NC) > kChipMost || E > C * most_lines(V, P, a.early)) return 0;  // fewer blocks hold less
+        if (bytes(c, V, ms, a.want_post, NC) > kChipMost || E > C * most_lines(c, V, P, a.early)) return 0;  // fewer blocks hold less
         if ((C - 1) * NC >= c.N) continue;  // a block would have no variable
         const auto key = std::make_pair(kernel, C);
         auto f = active.find(key);
