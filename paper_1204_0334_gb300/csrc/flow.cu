@@ -95,11 +95,26 @@ static uint32_t fill_code(const QcDesc &d, int FV, Code &c) {
     return std::max(c.J * c.rch1.d + (uint32_t)c.nsyn, c.L * c.vch.d);  // tiles of the largest phase
 }
 
-// the code table's entry, an empty log, every slot with its first package and its pack phase open
+// the code table's entry, an empty log, every slot with its first package and its pack phase open; the
+// log by all blocks, the rest by the first
+constexpr int kStartEntries = 4096;  // entries a block
 __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args a) {
+    const int kind = a.sim ? F_SYN : F_PACK;
+    for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < a.log_len; n += gridDim.x * blockDim.x) {
+        Entry e;
+        if (n < a.W) {
+            e.w0 = entry_w0(kind, 0, a.sim ? 0 : 1, 0, a.sim ? 0 : n);
+            e.w1 = entry_w1((uint32_t)n, n, (uint32_t)(((long long)n * st.tiles) % a.blocks), (uint32_t)st.tiles);
+        } else {
+            e.w0 = 0ull;
+            e.w1 = entry_w1((uint32_t)(n - a.log_len), 0, 0u, 0u);  // the sequence number of the lap before
+        }
+        a.log[n] = e;
+    }
+    if (blockIdx.x) return;
     const int *src = reinterpret_cast<const int *>(&st.code);
     int *dst = reinterpret_cast<int *>(a.codes);
-    const int V = st.V, kind = a.sim ? F_SYN : F_PACK;
+    const int V = st.V;
     if (a.sim) {
         if (threadIdx.x == 0) *a.sim = st.sim;
         for (int i = threadIdx.x; i < a.W * 128; i += blockDim.x) {
@@ -114,17 +129,6 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
         a.ctl->next = a.W;
         a.ctl->live = a.W;
         a.ctl->abort = 0;
-    }
-    for (int n = threadIdx.x; n < kLog; n += blockDim.x) {
-        Entry e;
-        if (n < a.W) {
-            e.w0 = entry_w0(kind, 0, a.sim ? 0 : 1, 0, a.sim ? 0 : n);
-            e.w1 = entry_w1((uint32_t)n, n, (uint32_t)(((long long)n * st.tiles) % a.blocks), (uint32_t)st.tiles);
-        } else {
-            e.w0 = 0ull;
-            e.w1 = entry_w1((uint32_t)n - kLog, 0, 0u, 0u);  // the sequence number of the lap before
-        }
-        a.log[n] = e;
     }
     const int s = threadIdx.x;
     if (s >= a.W) return;
@@ -141,7 +145,7 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
 }
 
 ldpc_status start(const Args &a, const Start &st, cudaStream_t s) {
-    start_kernel<<<1, 1024, 0, s>>>(st, a);
+    start_kernel<<<(a.log_len + kStartEntries - 1) / kStartEntries, 1024, 0, s>>>(st, a);
     count_launch();
     LDPC_CUDA_TRY(cudaGetLastError());
     return LDPC_OK;
@@ -151,8 +155,16 @@ ldpc_status start(const Args &a, const Start &st, cudaStream_t s) {
 
 using namespace flow;
 
-size_t flow_ctl_bytes(int W) {
-    return (size_t)W * sizeof(Slot) + 256 + kLog * sizeof(Entry) + sizeof(Code);
+size_t flow_ctl_bytes(int W, int log_cap) {
+    return (size_t)W * sizeof(Slot) + 256 + (size_t)log_cap * sizeof(Entry) + sizeof(Code);
+}
+
+// blocks a launch may have on this device (one an SM)
+static int flow_blocks() {
+    int dev = 0, sms = 0;
+    cudaGetDevice(&dev);
+    cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+    return std::max(1, std::min(sms, 1 << kLogBase));
 }
 
 void flow_slot_bytes(const QcDesc &d, int msg, int algo, bool post, size_t *b4) {
@@ -227,9 +239,10 @@ static ldpc_status prepare(const QcDesc &d, const FlowMem &m, const ldpc_decode_
     a.slots = (Slot *)m.ctl;
     a.ctl = (Ctl *)((char *)m.ctl + (size_t)m.W * sizeof(Slot));
     a.log = (Entry *)((char *)a.ctl + 256);
-    a.codes = (Code *)(a.log + kLog);
+    a.codes = (Code *)(a.log + m.log_cap);
     a.ncodes = 1;
-    a.W = W;
+    a.most_blocks = flow_blocks();
+    a.W = std::min(W, log_slots(m.log_cap, a.most_blocks));
     a.msg = (uint32_t *)m.msg, a.mu = (uint32_t *)m.mu, a.post = (float *)m.post, a.hw = (uint32_t *)m.hw;
     a.msg_stride = b[0] / 4, a.mu_stride = b[1] / 4, a.post_stride = b[2] / 4, a.hw_stride = b[3] / 4;
     a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post;
@@ -277,6 +290,7 @@ struct ldpc_flow_ws {
     size_t cap[4] = {0, 0, 0, 0};
     void *buf[4] = {nullptr, nullptr, nullptr, nullptr};
     void *ctl = nullptr, *sim = nullptr;  // sim: the simulation's state and its slots' frames
+    int log_cap = 0;
     int *err = nullptr;                   // pinned, device-mapped
     unsigned long long *host = nullptr;   // pinned copy of the simulation's counters
 };
@@ -305,9 +319,16 @@ static ldpc_status flow_ensure(ldpc_code c, int msg, int algo, bool post, int W,
         if (!c->flow) return fail(0);
     }
     ldpc_flow_ws &w = *c->flow;
-    if (!w.ctl && cudaMalloc(&w.ctl, flow_ctl_bytes(kMaxSlots)) != cudaSuccess) {
-        w.ctl = nullptr;
-        return fail(flow_ctl_bytes(kMaxSlots));
+    const int log_cap = std::min(log_entries(W, flow_blocks()), kMaxLog);
+    if (log_cap > w.log_cap) {
+        if (w.ctl) LDPC_CUDA_TRY(cudaDeviceSynchronize());
+        cudaFree(w.ctl);
+        w.log_cap = 0;
+        if (cudaMalloc(&w.ctl, flow_ctl_bytes(kMaxSlots, log_cap)) != cudaSuccess) {
+            w.ctl = nullptr;
+            return fail(flow_ctl_bytes(kMaxSlots, log_cap));
+        }
+        w.log_cap = log_cap;
     }
     if (!w.err) {
         if (cudaHostAlloc((void **)&w.err, 64, cudaHostAllocMapped) != cudaSuccess) {
@@ -354,7 +375,7 @@ ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldp
     const ldpc_status e = flow_ensure(c, o.msg, o.algo, post != nullptr, W, false);
     if (e != LDPC_OK) return e;
     const ldpc_flow_ws &w = *c->flow;
-    FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.err};
+    FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.log_cap, w.err};
     return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
 }
 
@@ -365,7 +386,7 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
     ldpc_status e = flow_ensure(c, o.msg, o.algo, false, W, true);
     if (e != LDPC_OK) return e;
     ldpc_flow_ws &w = *c->flow;
-    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.err};
+    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.log_cap, w.err};
     std::memset(h, 0, 8 * sizeof(*h));
     constexpr int64_t kMost = (int64_t)1 << 20;  // frames a launch, so that none runs for minutes
     for (int64_t at = 0; at < max_frames; at += kMost) {

@@ -721,7 +721,7 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
     for (int tries = 0;;) {
         if (!pl.loaded || pl.n - pl.first >= 32u) {
             pl.first = pl.n;
-            ld_entry(a.log + ((pl.n + lane) & (kLog - 1)), pl.w0, pl.w1);
+            ld_entry(a.log + ((pl.n + lane) & (uint32_t)(a.log_len - 1)), pl.w0, pl.w1);
             pl.loaded = true;
         }
         const int at = (int)(pl.n - pl.first);
@@ -742,7 +742,7 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
             continue;
         }
         if (ahead < (SEQ >> 1)) {
-            ++pl.n;  // overwritten: it was finished without this block
+            ++pl.n;  // overwritten: it had no tile of this block's (log_entries)
             continue;
         }
         // not opened yet
@@ -782,7 +782,7 @@ __device__ __forceinline__ void open_phase(const Args &a, Slot &sl, int slot, co
     const unsigned long long t = atomicAdd(&a.ctl->tail, (1ull << 40) | tiles);
     const uint32_t n = (uint32_t)(t >> 40), base = (uint32_t)((t & ((1ull << 40) - 1ull)) % gridDim.x);
     __threadfence();
-    st_entry(a.log + (n & (kLog - 1)), entry_w0(kind, stop, it, code, pk), entry_w1(n, slot, base, tiles));
+    st_entry(a.log + (n & (uint32_t)(a.log_len - 1)), entry_w0(kind, stop, it, code, pk), entry_w1(n, slot, base, tiles));
 }
 
 // the slot's next package, or the end (one lane)
@@ -1294,7 +1294,8 @@ static ldpc_status launch(Args &a, const Start &st, int tiles, cudaStream_t s) {
         set_error("the flow kernel does not fit an SM (%zu bytes of shared memory)", smem);
         return LDPC_ECUDA;
     }
-    a.blocks = std::min({tiles, most, 1 << kLogBase});
+    a.blocks = std::min({tiles, most, a.most_blocks});
+    a.log_len = log_entries(a.W, a.blocks);
     const ldpc_status e = start(a, st, s);
     if (e != LDPC_OK) return e;
     // cooperative: all blocks resident or none, whatever else runs on the device

@@ -14,7 +14,7 @@ constexpr int kStages = 3;                          // tiles a block holds: in w
 constexpr int kThreads = (kComputeWarps + 1 + kStages) * 32;  // and the taking warp, a retiring warp per stage
 constexpr int kLookLimit = 1 << 24;                 // looks for a new phase before a block gives up (seconds)
 constexpr int kMaxSlots = 256;
-constexpr int kLog = 4096;                          // entries of the phase log (a power of two)
+constexpr int kMaxLog = 1 << 16;                    // entries of the longest phase log
 // check rows of a tile: one a compute warp (two of short rows; fewer of 32-edge rows, so that three
 // tiles fit in shared memory)
 __host__ __device__ constexpr int tile_rows(int J, int L) {
@@ -63,6 +63,21 @@ __host__ __device__ inline unsigned long long entry_w1(uint32_t seq, int slot, u
     return x << kLogTiles | tiles;
 }
 
+// Entries of the phase log, a power of two.  Entry n is overwritten by entry n + length, which must not be
+// opened while some block b has a tile of entry n that it has not read.  Tiles are numbered as they are
+// opened and tile t belongs to block t mod blocks, so every `blocks` consecutive tiles hold one of b's.
+// b reads the log in order: a phase opened after n with a tile of b does not end before b has read n, and
+// its slot opens no other.  With entry n that is at most one such phase a slot, so at most slots * blocks
+// tiles, and as many phases, are opened from entry n on (each has a tile but the last of all, which is
+// opened when no slot has a phase left).
+inline int log_entries(int slots, int blocks) {
+    int n = 64;  // more than the 32 entries that are looked at together
+    while (n < (long long)slots * blocks + 1) n *= 2;
+    return n;
+}
+// slots that a log of `entries` serves
+inline int log_slots(int entries, int blocks) { return (entries - 1) / blocks; }
+
 // a package in work
 struct alignas(64) Slot {
     unsigned int done, syn_done;  // finished tiles of the open phase, finished syndrome tiles
@@ -105,13 +120,14 @@ struct Args {
     Slot *slots;
     Ctl *ctl;
     Entry *log;
+    int log_len;               // its entries (a power of two)
     int W, P;                  // slots, packages
     uint32_t *msg, *mu, *hw;   // per slot: [E][32], [N][32 FV], [N][V]
     float *post;               // per slot: [N][32 V]
     size_t msg_stride, mu_stride, hw_stride, post_stride;  // words
     int max_iter, early, want_post;
     int split;                 // the early-stop syndrome is a phase of its own
-    int blocks;
+    int blocks, most_blocks;   // of the launch; as many as the log allows
     float clip, qscale, lsb;
     const int *pkg_code;       // package -> code (NULL: one code)
     Sim *sim;                  // refill mode, else NULL
@@ -148,10 +164,10 @@ constexpr int kErrVars = 128 * kComputeWarps;  // variables of a tile that count
 struct FlowMem {
     void *msg, *mu, *post, *hw;  // W slots each
     void *ctl;                   // flow_ctl_bytes()
-    int W;
+    int W, log_cap;              // slots, entries of the phase log
     int *err;
 };
-size_t flow_ctl_bytes(int W);
+size_t flow_ctl_bytes(int W, int log_cap);
 // slots a decode of P packages keeps in work, and the bytes of one slot's buffers
 int flow_slots(const QcDesc &d, int msg, int algo, bool post, int P);
 void flow_slot_bytes(const QcDesc &d, int msg, int algo, bool post, size_t *b4);

@@ -32,9 +32,9 @@ constexpr size_t kNoallocBytes = (size_t)16 << 20;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
-// the flow decoder's slots and code table (not part of the 16 MiB that bound a request)
+// the flow decoder's slots, phase log and code table (not part of the 16 MiB that bound a request)
 static __device__ __align__(256) unsigned char g_noalloc_ctl[flow::kMaxSlots * sizeof(flow::Slot) + 256 +
-                                                             flow::kLog * sizeof(flow::Entry) + sizeof(flow::Code)];
+                                                             flow::kMaxLog * sizeof(flow::Entry) + sizeof(flow::Code)];
 
 namespace {
 constexpr int kMaxDevices = 64;
@@ -140,7 +140,7 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
         flow_slot_bytes(c->d, o.msg, o.algo, post != nullptr, b);
         const int W = std::min((gamma + 32 * V - 1) / (32 * V), flow::kMaxSlots);
         for (int i = 0; i < 4; ++i) at[i] = x, x += b[i] * W;
-        const FlowMem m{base + at[0], base + at[1], base + at[2], base + at[3], ctl, W, err};
+        const FlowMem m{base + at[0], base + at[1], base + at[2], base + at[3], ctl, W, flow::kMaxLog, err};
         return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
     }
     // A private view of the code object whose workspace points into the scratch.  It

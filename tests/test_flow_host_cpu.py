@@ -1,0 +1,71 @@
+"""The flow decoder's host part on a machine without a GPU (fake_device.py): what its launches are given,
+what it allocates and when, and what a caller is told when a device-side wait gives up."""
+import pytest
+
+from fake_device import FakeDevice
+
+
+@pytest.fixture(scope="module")
+def built(tmp_path_factory):
+    return FakeDevice(tmp_path_factory.mktemp("fake"))
+
+
+@pytest.fixture
+def dev(built):
+    built.reset()
+    return built
+
+
+def phases_while_one_block_waits(slots, blocks, cycle):
+    """Phases that can be open or done from the one on whose tile a block is held up, all other blocks being
+    done with theirs at once: tile t of all belongs to block t mod blocks, a slot goes through the phases
+    of `cycle` (tiles each), and stops at the first that has a tile of the held-up block."""
+    opened = tiles = 0
+    at = [0] * slots
+    running = list(range(slots))
+    while running:
+        still = []
+        for s in running:
+            n = cycle[at[s] % len(cycle)]
+            first = -tiles % blocks  # the phase's first tile of block 0
+            tiles += n
+            opened += 1
+            at[s] += 1
+            if first >= n:
+                still.append(s)
+        running = still
+    return opened
+
+
+# J, L, p: the shortest codes (a tile or a few a phase), short ones on many slots, longer ones on few
+@pytest.mark.parametrize("J,L,p", [(1, 2, 1), (2, 6, 20), (3, 6, 64), (4, 12, 31), (4, 12, 211), (4, 24, 100),
+                                   (4, 24, 765), (8, 32, 61)])
+@pytest.mark.parametrize("algo,msg", [(0, 0), (0, 1), (1, 2)])
+def test_phase_log_holds_what_a_late_block_has_not_read(dev, J, L, p, algo, msg):
+    """A log entry is not overwritten while a block may still have to read it, whatever the number of slots
+    and however long one block is held up."""
+    code = dev.code(J, L, p)
+    N = L * p
+    opts = dict(algo=algo, msg=msg, max_iter=20, early_stop=1)
+    seen = 0
+    for frames in (33, 300, 10000, 70000):
+        if frames * N <= 1 << 24:
+            assert dev.decode(code, N, frames, post=True, **opts) == 0
+    for slots in (64, 1024, 16384, 32768):
+        assert dev.sim(code, 5 * slots, slots, **opts) == 0
+    for f in dev.flows():
+        fewest = min(f["nsyn"], f["cn_tiles"], f["vn_tiles"], -(-N // 256))
+        for cycle in ([f["nsyn"], f["cn_tiles"], f["vn_tiles"]], [1], [fewest]):
+            assert phases_while_one_block_waits(f["W"], f["blocks"], cycle) < f["log_len"], f
+        seen = max(seen, f["W"])
+    if msg and N < 1000:
+        assert seen == 256  # the most slots there are
+    dev.c.ldpc_code_destroy(code)
+
+
+def test_phase_log_of_the_allocation_free_decode(dev):
+    code = dev.code(2, 4, 20)
+    assert dev.decode(code, 80, 256 * 32, noalloc=True, max_iter=9, early_stop=1) == 0
+    (f,) = dev.flows()
+    assert f["W"] == 256 and f["log_len"] > phases_while_one_block_waits(f["W"], f["blocks"], [1])
+    dev.c.ldpc_code_destroy(code)

@@ -1,0 +1,45 @@
+"""The flow decoder on calls that are seen to reach it (two launches, whatever the iterations): as many
+packages in work as there are slots, against the same frames decoded by themselves."""
+import pytest
+
+import synth
+from test_gpu_flow import pkg, setup  # noqa: F401  (the module's fixture)
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+
+def launches(pkg, call):
+    pkg.ldpc_profile_enable(False)  # clears the count
+    out = call()
+    return out, pkg.ldpc_profile_read()["launches"]
+
+
+@pytest.mark.parametrize("algo,msg,slots", [(0, 1, 16384), (1, 2, 32768)])
+def test_simulation_on_256_packages(pkg, algo, msg, slots):
+    """A short code's simulation on the most slots there are counts what a batch decode of its frames counts."""
+    code = pkg.QCCode(synth.qc_shifts(3, 6, 64, seed=8), 64)
+    frames = 2 * slots + 77
+    kw = dict(max_iter=14, early_stop=1, algo=algo, msg=msg)
+    r, n = launches(pkg, lambda: code.ber_sim(2.0, seed=11, first_frame=5, max_frames=frames,
+                                              target_frame_errors=1 << 40, gamma=slots, **kw))
+    assert n == 2
+    llr = code.channel(2.0, 11, 5, frames)
+    _, hard, it, ok = code.decode(llr, want_post=False, **kw)
+    e = hard.sum(dim=1).long()
+    assert r["frames"] == frames and r["iters_sum"] == int(it.sum())
+    assert r["bit_errors"] == int(e.sum()) and r["frame_errors"] == int((e > 0).sum())
+    assert r["bit_errors_sq"] == int((e * e).sum()) and r["undetected"] == int(((e > 0) & (ok == 1)).sum())
+
+
+def test_decode_of_more_packages_than_slots(pkg):
+    """282 packages of a small code, 256 in work at once."""
+    code, _, _ = setup(pkg, 2, 4, 20, 0, 7)
+    mu = torch.from_numpy(synth.gaussian_llrs(9000, code.N, seed=3, ebn0_db=2.0, rate=0.5)).cuda()
+    whole, n = launches(pkg, lambda: code.decode(mu, max_iter=12, early_stop=True))
+    assert n == 2
+    for f in range(0, 9000, 3000):
+        part, n = launches(pkg, lambda: code.decode(mu[f:f + 3000], max_iter=12, early_stop=True))
+        assert n == 1  # on chip
+        for a, b in zip(whole, part):
+            assert torch.equal(a[f:f + 3000], b)
