@@ -17,19 +17,29 @@ def launches(pkg, call):
 
 @pytest.mark.parametrize("algo,msg,slots", [(0, 1, 16384), (1, 2, 32768)])
 def test_simulation_on_256_packages(pkg, algo, msg, slots):
-    """A short code's simulation on the most slots there are counts what a batch decode of its frames counts."""
+    """A short code's simulation on the most slots there are counts what the simulation by a launch a step
+    counts on the same frames (a target that can be met, and is not), and with integer messages what a batch
+    decode of them counts (binary16 messages start from rounded channel values there, from FP32 in a batch)."""
     code = pkg.QCCode(synth.qc_shifts(3, 6, 64, seed=8), 64)
     frames = 2 * slots + 77
     kw = dict(max_iter=14, early_stop=1, algo=algo, msg=msg)
-    r, n = launches(pkg, lambda: code.ber_sim(2.0, seed=11, first_frame=5, max_frames=frames,
-                                              target_frame_errors=1 << 40, gamma=slots, **kw))
+
+    def sim(target):
+        r, n = launches(pkg, lambda: code.ber_sim(2.0, seed=11, first_frame=5, max_frames=frames,
+                                                  target_frame_errors=target, gamma=slots, **kw))
+        r.pop("seconds")
+        return r, n
+
+    r, n = sim(1 << 40)
     assert n == 2
-    llr = code.channel(2.0, 11, 5, frames)
-    _, hard, it, ok = code.decode(llr, want_post=False, **kw)
-    e = hard.sum(dim=1).long()
-    assert r["frames"] == frames and r["iters_sum"] == int(it.sum())
-    assert r["bit_errors"] == int(e.sum()) and r["frame_errors"] == int((e > 0).sum())
-    assert r["bit_errors_sq"] == int((e * e).sum()) and r["undetected"] == int(((e > 0) & (ok == 1)).sum())
+    other, n = sim(frames)
+    assert n > 2 and r == other
+    if msg == 2:
+        _, hard, it, ok = code.decode(code.channel(2.0, 11, 5, frames), want_post=False, **kw)
+        e = hard.sum(dim=1).long()
+        assert r["frames"] == frames and r["iters_sum"] == int(it.sum())
+        assert r["bit_errors"] == int(e.sum()) and r["frame_errors"] == int((e > 0).sum())
+        assert r["bit_errors_sq"] == int((e * e).sum()) and r["undetected"] == int(((e > 0) & (ok == 1)).sum())
 
 
 def test_decode_of_more_packages_than_slots(pkg):
