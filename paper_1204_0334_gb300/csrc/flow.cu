@@ -95,7 +95,7 @@ static uint32_t fill_code(const QcDesc &d, int FV, Code &c) {
     return std::max(c.J * c.rch1.d + (uint32_t)c.nsyn, c.L * c.vch.d);  // tiles of the largest phase
 }
 
-// the code table's entry, an empty log, every slot with its first package and its pack phase open; the
+// the code's entry, an empty log, every slot with its first package and its pack phase open; the
 // log by all blocks, the rest by the first
 constexpr int kStartEntries = 4096;  // entries a block
 __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args a) {
@@ -103,7 +103,7 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
     for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < a.log_len; n += gridDim.x * blockDim.x) {
         Entry e;
         if (n < a.W) {
-            e.w0 = entry_w0(kind, 0, a.sim ? 0 : 1, 0, a.sim ? 0 : n);
+            e.w0 = entry_w0(kind, 0, a.sim ? 0 : 1, a.sim ? 0 : n);
             e.w1 = entry_w1((uint32_t)n, n, (uint32_t)(((long long)n * st.tiles) % a.blocks), (uint32_t)st.tiles);
         } else {
             e.w0 = 0ull;
@@ -113,7 +113,7 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
     }
     if (blockIdx.x) return;
     const int *src = reinterpret_cast<const int *>(&st.code);
-    int *dst = reinterpret_cast<int *>(a.codes);
+    int *dst = reinterpret_cast<int *>(a.code);
     const int V = st.V;
     if (a.sim) {
         if (threadIdx.x == 0) *a.sim = st.sim;
@@ -239,8 +239,7 @@ static ldpc_status prepare(const QcDesc &d, const FlowMem &m, const ldpc_decode_
     a.slots = (Slot *)m.ctl;
     a.ctl = (Ctl *)((char *)m.ctl + (size_t)m.W * sizeof(Slot));
     a.log = (Entry *)((char *)a.ctl + 256);
-    a.codes = (Code *)(a.log + m.log_cap);
-    a.ncodes = 1;
+    a.code = (Code *)(a.log + m.log_cap);
     a.most_blocks = flow_blocks();
     a.W = std::min(W, log_slots(m.log_cap, a.most_blocks));
     a.msg = (uint32_t *)m.msg, a.mu = (uint32_t *)m.mu, a.post = (float *)m.post, a.hw = (uint32_t *)m.hw;

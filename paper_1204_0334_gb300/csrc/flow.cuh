@@ -31,16 +31,6 @@ __device__ __forceinline__ bool mbar_try(uint32_t bar, uint32_t parity) {
         : "memory");
     return ok != 0u;
 }
-// the same without suspending the thread
-__device__ __forceinline__ bool mbar_test(uint32_t bar, uint32_t parity) {
-    uint32_t ok;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.test_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(ok)
-        : "r"(bar), "r"(parity)
-        : "memory");
-    return ok != 0u;
-}
 constexpr int kWaitLimit = 1 << 23;  // tries of one wait (each suspends up to the hardware's time limit)
 __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity) {
     for (int i = 0; i < kWaitLimit; ++i)
@@ -106,7 +96,7 @@ struct Cfg {
 };
 
 struct Desc {
-    int kind, rows, j, first, n0, code, slot, pk, it, post, stop;
+    int kind, rows, j, first, n0, slot, pk, it, post, stop;
     uint32_t pm, tiles;
     uint32_t dn[4];
 };
@@ -120,7 +110,7 @@ struct Smem {
     uint8_t list[kStages][32 * V];  // channel tile: the package's frames that enter, and their ids
     uint32_t fid[kStages][32 * V];  // (less the launch's first)
     uint32_t hw[kStages][4 * kComputeWarps * V];  // variable tile: the decisions so far (where frames have stopped)
-    Code code;                                     // the code of a flow of one code
+    Code code;
     alignas(8) unsigned long long full[kStages], used[kStages], empty[kStages];
 };
 
@@ -759,8 +749,8 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
 
 // opens a slot's next phase (one lane)
 template <typename C>
-__device__ __forceinline__ void open_phase(const Args &a, Slot &sl, int slot, const Code &c, int code, int pk, int kind,
-                                           int it, int stop) {
+__device__ __forceinline__ void open_phase(const Args &a, Slot &sl, int slot, const Code &c, int pk, int kind, int it,
+                                           int stop) {
     uint32_t tiles = 0;
     switch (kind) {
         case F_CN:
@@ -782,38 +772,34 @@ __device__ __forceinline__ void open_phase(const Args &a, Slot &sl, int slot, co
     const unsigned long long t = atomicAdd(&a.ctl->tail, (1ull << 40) | tiles);
     const uint32_t n = (uint32_t)(t >> 40), base = (uint32_t)((t & ((1ull << 40) - 1ull)) % gridDim.x);
     __threadfence();
-    st_entry(a.log + (n & (uint32_t)(a.log_len - 1)), entry_w0(kind, stop, it, code, pk), entry_w1(n, slot, base, tiles));
+    st_entry(a.log + (n & (uint32_t)(a.log_len - 1)), entry_w0(kind, stop, it, pk), entry_w1(n, slot, base, tiles));
 }
 
 // the slot's next package, or the end (one lane)
 template <typename C, int V>
-__device__ __forceinline__ void next_package(const Args &a, Slot &sl, int slot) {
+__device__ __forceinline__ void next_package(const Args &a, const Code &c, Slot &sl, int slot) {
     const int g = atomicAdd(&a.ctl->next, 1);
     if (g >= a.P) {
         __threadfence();
-        if (atomicSub(&a.ctl->live, 1) == 1) open_phase<C>(a, sl, slot, a.codes[0], 0, 0, F_EXIT, 0, 0);
+        if (atomicSub(&a.ctl->live, 1) == 1) open_phase<C>(a, sl, slot, c, 0, F_EXIT, 0, 0);
         return;
     }
-    const int code = a.pkg_code ? a.pkg_code[g] : 0;
-    const Code &c = a.codes[code];
-    const int pk = g - c.pk0;
     uint32_t stop = 0u;
     sl.all = 0;
     for (int v = 0; v < V; ++v) {
-        const int n = c.gamma - pk * C::W - v;  // frames v, V + v, ... of the package
+        const int n = c.gamma - g * C::W - v;  // frames v, V + v, ... of the package
         const int lanes = n <= 0 ? 0 : min(32, (n + V - 1) / V);
         const uint32_t valid = lanes == 32 ? 0xffffffffu : (1u << lanes) - 1u;
         sl.dn[v] = ~valid;
         sl.un[v] = 0u;
         stop |= ~valid;
     }
-    open_phase<C>(a, sl, slot, c, code, pk, F_PACK, 1, stop != 0u);
+    open_phase<C>(a, sl, slot, c, g, F_PACK, 1, stop != 0u);
 }
-
 
 // what finish() needs of a tile
 struct Fin {
-    int kind, code, slot, pk, it, stop;
+    int kind, slot, pk, it, stop;
     uint32_t tiles;
 };
 
@@ -913,9 +899,9 @@ __device__ __forceinline__ void tally(const Args &a, Slot &sl, SimSlot &ss, int 
 
 // a slot has no frame left (one lane)
 template <typename C>
-__device__ __forceinline__ void end_slot(const Args &a, Slot &sl, int slot) {
+__device__ __forceinline__ void end_slot(const Args &a, const Code &c, Slot &sl, int slot) {
     __threadfence();
-    if (atomicSub(&a.ctl->live, 1) == 1) open_phase<C>(a, sl, slot, a.codes[0], 0, 0, F_EXIT, 0, 0);
+    if (atomicSub(&a.ctl->live, 1) == 1) open_phase<C>(a, sl, slot, c, 0, F_EXIT, 0, 0);
 }
 
 // finish() in refill mode: syndrome, check and variable phases in turn
@@ -932,17 +918,17 @@ __device__ __forceinline__ void finish_refill(const Args &a, const Code &c, cons
         const int what = refill<C, V>(a, sl, ss, lane);
         __syncwarp();  // opening the phase publishes what the lanes wrote
         if (lane == 0) {
-            if (what) open_phase<C>(a, sl, d.slot, c, 0, 0, F_CN, what, 0);
-            else end_slot<C>(a, sl, d.slot);
+            if (what) open_phase<C>(a, sl, d.slot, c, 0, F_CN, what, 0);
+            else end_slot<C>(a, c, sl, d.slot);
         }
     } else if (d.kind == F_VN) {
-        if (lane == 0) open_phase<C>(a, sl, d.slot, c, 0, 0, F_SYN, 0, 0);
+        if (lane == 0) open_phase<C>(a, sl, d.slot, c, 0, F_SYN, 0, 0);
     } else {
         if ((d.it & 1) && !a.sim->io) tally<V>(a, sl, ss, lane);
         __syncwarp();
         if (lane == 0) {
-            if (d.it & 4) open_phase<C>(a, sl, d.slot, c, 0, 0, F_VN, 0, 0);
-            else end_slot<C>(a, sl, d.slot);
+            if (d.it & 4) open_phase<C>(a, sl, d.slot, c, 0, F_VN, 0, 0);
+            else end_slot<C>(a, c, sl, d.slot);
         }
     }
     __syncwarp();
@@ -1007,8 +993,8 @@ __device__ __forceinline__ void finish(const Args &a, const Code &c, const Fin &
             default: break;
         }
         if (nk == F_OUT && !outs) nk = -1;
-        if (nk >= 0) open_phase<C>(a, sl, d.slot, c, d.code, d.pk, nk, it, stop);
-        else next_package<C, V>(a, sl, d.slot);
+        if (nk >= 0) open_phase<C>(a, sl, d.slot, c, d.pk, nk, it, stop);
+        else next_package<C, V>(a, c, sl, d.slot);
     }
     __syncwarp();
 }
@@ -1042,9 +1028,9 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
         }
         int kind = (int)bits(pl.e0, 0, 3), it = (int)bits(pl.e0, 4, kLogIt);
         const bool stop = bits(pl.e0, 3, 1) != 0u;
-        const int code = (int)bits(pl.e0, 4 + kLogIt, kLogCode), pk = (int)bits(pl.e0, 4 + kLogIt + kLogCode, kLogPk);
+        const int pk = (int)bits(pl.e0, 4 + kLogIt, kLogPk);
         const int slot = (int)bits(pl.e1, kLogTiles + kLogBase, kLogSlot);
-        const Code &c = a.ncodes == 1 ? sm.code : a.codes[code];
+        const Code &c = sm.code;
         if (kind == F_FIN) {
             kind = F_SYN;
             it = -1;
@@ -1060,7 +1046,6 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
         }
         if (lane == 0) {
             d.kind = kind;
-            d.code = code;
             d.slot = slot;
             d.pk = pk;
             d.it = it;
@@ -1179,8 +1164,8 @@ __device__ __forceinline__ void retiring_warp(const Args &a, SM &sm, int st, int
         const Desc &d = sm.desc[st];
         const int kind = d.kind;
         if (kind == F_EXIT) return;
-        const Fin n{kind, d.code, d.slot, d.pk, d.it, d.stop, d.tiles};
-        const Code &c = a.ncodes == 1 ? sm.code : a.codes[n.code];
+        const Fin n{kind, d.slot, d.pk, d.it, d.stop, d.tiles};
+        const Code &c = sm.code;
         if (kind == F_CN || kind == F_VN) {
             char *msg = reinterpret_cast<char *>(a.msg + (size_t)d.slot * a.msg_stride);
             const uint32_t src = smem_u32(sm.stage[st] + lane * (kind == F_CN ? C::ROWS : C::KC) * 32);
@@ -1230,11 +1215,9 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const Args a) {
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
         fence_async();
     }
-    if (a.ncodes == 1) {
-        const int *src = reinterpret_cast<const int *>(a.codes);
-        int *dst = reinterpret_cast<int *>(&sm.code);
-        for (int i = threadIdx.x; i < (int)(sizeof(Code) / 4); i += blockDim.x) dst[i] = src[i];
-    }
+    const int *src = reinterpret_cast<const int *>(a.code);
+    int *dst = reinterpret_cast<int *>(&sm.code);
+    for (int i = threadIdx.x; i < (int)(sizeof(Code) / 4); i += blockDim.x) dst[i] = src[i];
     __syncthreads();
     if (warp == kComputeWarps) return taking_warp<C, JX, V>(a, sm, lane);
     if (warp > kComputeWarps) return retiring_warp<C, V>(a, sm, warp - kComputeWarps - 1, lane);
@@ -1250,7 +1233,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const Args a) {
         const int kind = d.kind;
         uint32_t *stage = sm.stage[st];
         const size_t slot = (size_t)d.slot;
-        const Code &c = a.ncodes == 1 ? sm.code : a.codes[d.code];
+        const Code &c = sm.code;
         if (kind == F_CN) {
             const float2 *prm = nullptr;
             if constexpr (RULE == kFlowNOMS) {

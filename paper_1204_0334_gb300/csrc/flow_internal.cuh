@@ -27,13 +27,13 @@ enum { kFlowSP = 0, kFlowMS = 1, kFlowNOMS = 2 };
 // phases; F_SYN is also a tile of F_CN and F_FIN, the last three are tiles of F_CN in refill mode
 enum { F_PACK = 0, F_CN, F_VN, F_FIN, F_OUT, F_SYN, F_EXIT, F_ERR, F_ROWS, F_CHAN };
 
-// one code of a flow and the caller's buffers of its frames
+// the code of a launch and the caller's buffers of its frames
 struct Code {
     int J, L, p, N, M;
     int kc;                  // variables of a variable tile (a multiple of 4)
     int nsyn;                // syndrome tiles
     FastDiv divp, rch, rch1, vch;  // p; check tiles per block row (later / first iteration); variable tiles per column
-    int pk0, gamma;          // first package of the flow that is this code's, frames
+    int gamma;               // frames
     const float *llr;
     float *post;
     uint8_t *hard;
@@ -43,15 +43,14 @@ struct Code {
 };
 
 // A phase that has been opened, 16 bytes written and read at once.  w0: kind (3 bits), frames stopped
-// (1), iteration (17), code (12), package (26).  w1: tiles (24), the number of tiles opened before it
+// (1), iteration (17), package (26).  w1: tiles (24), the number of tiles opened before it
 // modulo the blocks (10), slot (8), sequence number (22).
-constexpr int kLogIt = 17, kLogCode = 12, kLogPk = 26, kLogTiles = 24, kLogBase = 10, kLogSlot = 8, kLogSeq = 22;
+constexpr int kLogIt = 17, kLogPk = 26, kLogTiles = 24, kLogBase = 10, kLogSlot = 8, kLogSeq = 22;
 struct alignas(16) Entry {
     unsigned long long w0, w1;
 };
-__host__ __device__ inline unsigned long long entry_w0(int kind, int stop, int it, int code, int pk) {
+__host__ __device__ inline unsigned long long entry_w0(int kind, int stop, int it, int pk) {
     unsigned long long x = (unsigned)pk;
-    x = x << kLogCode | (unsigned)code;
     x = x << kLogIt | (unsigned)it;
     x = x << 1 | (unsigned)stop;
     return x << 3 | (unsigned)kind;
@@ -115,8 +114,7 @@ struct Ctl {
 };
 
 struct Args {
-    Code *codes;
-    int ncodes;
+    Code *code;
     Slot *slots;
     Ctl *ctl;
     Entry *log;
@@ -129,7 +127,6 @@ struct Args {
     int split;                 // the early-stop syndrome is a phase of its own
     int blocks, most_blocks;   // of the launch; as many as the log allows
     float clip, qscale, lsb;
-    const int *pkg_code;       // package -> code (NULL: one code)
     Sim *sim;                  // refill mode, else NULL
     SimSlot *simslots;
     int *err;                  // host word set when a wait ran out

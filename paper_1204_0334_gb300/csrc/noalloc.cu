@@ -32,7 +32,7 @@ constexpr size_t kNoallocBytes = (size_t)16 << 20;
 
 static __device__ __align__(256) unsigned char g_noalloc_scratch[kNoallocBytes];
 
-// the flow decoder's slots, phase log and code table (not part of the 16 MiB that bound a request)
+// the flow decoder's slots, phase log and code (not part of the 16 MiB that bound a request)
 static __device__ __align__(256) unsigned char g_noalloc_ctl[flow::kMaxSlots * sizeof(flow::Slot) + 256 +
                                                              flow::kMaxLog * sizeof(flow::Entry) + sizeof(flow::Code)];
 
