@@ -103,11 +103,12 @@ __global__ void __launch_bounds__(1024) start_kernel(const Start st, const Args 
     for (int n = blockIdx.x * blockDim.x + threadIdx.x; n < a.log_len; n += gridDim.x * blockDim.x) {
         Entry e;
         if (n < a.W) {
-            e.w0 = entry_w0(kind, 0, a.sim ? 0 : 1, a.sim ? 0 : n);
+            e.w0 = entry_w0((uint32_t)n, kind, 0, a.sim ? 0 : 1, a.sim ? 0 : n);
             e.w1 = entry_w1((uint32_t)n, n, (uint32_t)(((long long)n * st.tiles) % a.blocks), (uint32_t)st.tiles);
         } else {
-            e.w0 = 0ull;
-            e.w1 = entry_w1((uint32_t)(n - a.log_len), 0, 0u, 0u);  // the sequence number of the lap before
+            const uint32_t before = (uint32_t)(n - a.log_len);  // the sequence number of the lap before
+            e.w0 = entry_w0(before, 0, 0, 0, 0);
+            e.w1 = entry_w1(before, 0, 0u, 0u);
         }
         a.log[n] = e;
     }

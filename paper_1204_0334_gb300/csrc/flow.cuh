@@ -697,8 +697,6 @@ __device__ __forceinline__ uint32_t bits(unsigned long long x, int at, int n) {
 // This block's next tile (its number in pl.idx - blocks, its phase in pl.e0, pl.e1); false: every
 // package is done (or the kernel gives up).
 __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_t &idx) {
-    constexpr uint32_t SEQ = (1u << kLogSeq) - 1u;
-    constexpr int kAtSeq = kLogTiles + kLogBase + kLogSlot;
     if (pl.idx != ~0u) {
         if (pl.idx < bits(pl.e1, 0, kLogTiles)) {
             idx = pl.idx;
@@ -717,8 +715,8 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
         const int at = (int)(pl.n - pl.first);
         pl.e0 = __shfl_sync(0xffffffffu, pl.w0, at);
         pl.e1 = __shfl_sync(0xffffffffu, pl.w1, at);
-        const uint32_t ahead = (bits(pl.e1, kAtSeq, kLogSeq) - pl.n) & SEQ;
-        if (ahead == 0u) {
+        const int is = entry_is(pl.e0, pl.e1, pl.n);
+        if (is == kEntryHere) {
             if (bits(pl.e0, 0, 3) == F_EXIT) return false;
             const uint32_t base = bits(pl.e1, kLogTiles, kLogBase);
             const uint32_t i = blockIdx.x >= base ? blockIdx.x - base : blockIdx.x + gridDim.x - base;
@@ -731,7 +729,7 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
             ++pl.n;  // none of its tiles is this block's
             continue;
         }
-        if (ahead < (SEQ >> 1)) {
+        if (is == kEntryPast) {
             ++pl.n;  // overwritten: it had no tile of this block's (log_entries)
             continue;
         }
@@ -772,7 +770,7 @@ __device__ __forceinline__ void open_phase(const Args &a, Slot &sl, int slot, co
     const unsigned long long t = atomicAdd(&a.ctl->tail, (1ull << 40) | tiles);
     const uint32_t n = (uint32_t)(t >> 40), base = (uint32_t)((t & ((1ull << 40) - 1ull)) % gridDim.x);
     __threadfence();
-    st_entry(a.log + (n & (uint32_t)(a.log_len - 1)), entry_w0(kind, stop, it, pk), entry_w1(n, slot, base, tiles));
+    st_entry(a.log + (n & (uint32_t)(a.log_len - 1)), entry_w0(n, kind, stop, it, pk), entry_w1(n, slot, base, tiles));
 }
 
 // the slot's next package, or the end (one lane)

@@ -42,24 +42,37 @@ struct Code {
     int sh[kMaxJ * kMaxL], eo[kMaxJ * kMaxL];  // [J][L]: shift (-1: zero block), first edge
 };
 
-// A phase that has been opened, 16 bytes written and read at once.  w0: kind (3 bits), frames stopped
-// (1), iteration (17), package (26).  w1: tiles (24), the number of tiles opened before it
-// modulo the blocks (10), slot (8), sequence number (22).
-constexpr int kLogIt = 17, kLogPk = 26, kLogTiles = 24, kLogBase = 10, kLogSlot = 8, kLogSeq = 22;
+// A phase that has been opened.  w0: kind (3 bits), frames stopped (1), iteration (17), package (26), sequence
+// number without its low five bits (17).  w1: tiles (24), the number of tiles opened before it modulo the
+// blocks (10), slot (8), sequence number (22).  The words are loaded and stored as a pair, which the memory
+// model takes for two accesses in no order: the entries that follow one another in a place are 64 or more
+// apart, so the numbers tell a new word from an old one.
+constexpr int kLogIt = 17, kLogPk = 26, kLogTiles = 24, kLogBase = 10, kLogSlot = 8, kLogSeq = 22, kLogLow = 5;
+constexpr uint32_t kLogMask = (1u << kLogSeq) - 1u;
 struct alignas(16) Entry {
     unsigned long long w0, w1;
 };
-__host__ __device__ inline unsigned long long entry_w0(int kind, int stop, int it, int pk) {
-    unsigned long long x = (unsigned)pk;
+__host__ __device__ inline unsigned long long entry_w0(uint32_t seq, int kind, int stop, int it, int pk) {
+    unsigned long long x = (seq & kLogMask) >> kLogLow;
+    x = x << kLogPk | (unsigned)pk;
     x = x << kLogIt | (unsigned)it;
     x = x << 1 | (unsigned)stop;
     return x << 3 | (unsigned)kind;
 }
 __host__ __device__ inline unsigned long long entry_w1(uint32_t seq, int slot, uint32_t base, uint32_t tiles) {
-    unsigned long long x = seq & ((1u << kLogSeq) - 1u);
+    unsigned long long x = seq & kLogMask;
     x = x << kLogSlot | (unsigned)slot;
     x = x << kLogBase | base;
     return x << kLogTiles | tiles;
+}
+// what two words read in entry n's place are: entry n, a later one that has overwritten it, or not (both of)
+// entry n yet
+enum { kEntryHere = 0, kEntryPast, kEntryAhead };
+__host__ __device__ inline int entry_is(unsigned long long w0, unsigned long long w1, uint32_t n) {
+    const uint32_t ahead = ((uint32_t)(w1 >> (kLogTiles + kLogBase + kLogSlot)) - n) & kLogMask;
+    if (ahead == 0u)
+        return (uint32_t)(w0 >> (4 + kLogIt + kLogPk)) == (n & kLogMask) >> kLogLow ? kEntryHere : kEntryAhead;
+    return ahead < (kLogMask >> 1) ? kEntryPast : kEntryAhead;
 }
 
 // Entries of the phase log, a power of two.  Entry n is overwritten by entry n + length, which must not be

@@ -69,3 +69,17 @@ def test_phase_log_of_the_allocation_free_decode(dev):
     (f,) = dev.flows()
     assert f["W"] == 256 and f["log_len"] > phases_while_one_block_waits(f["W"], f["blocks"], [1])
     dev.c.ldpc_code_destroy(code)
+
+
+@pytest.mark.parametrize("length", [64, 2048, 65536])
+def test_log_entry_read_in_two_parts(dev, length):
+    """A block that finds one word of an entry and the other of the entry before it in that place looks again,
+    whichever came first; words past the wrap of the sequence number too."""
+    here, past, ahead = 0, 1, 2
+    for n in (0, 5, length - 1, length, 12345, (1 << 22) - 1, 1 << 22, (1 << 22) + 77, (1 << 24) + 1, (1 << 32) - 3):
+        before, after = (n - length) % (1 << 32), (n + length) % (1 << 32)
+        assert dev.c.fake_entry_is(n, n, n) == here
+        assert dev.c.fake_entry_is(before, before, n) == ahead
+        assert dev.c.fake_entry_is(before, n, n) == ahead and dev.c.fake_entry_is(n, before, n) == ahead
+        assert dev.c.fake_entry_is(after, after, n) == past and dev.c.fake_entry_is(n, after, n) == past
+        assert dev.c.fake_entry_is(after, n, n) == ahead  # read again: n has been overwritten
