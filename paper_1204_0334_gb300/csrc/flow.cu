@@ -287,10 +287,11 @@ ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int
 // the workspace a code object keeps
 // ---------------------------------------------------------------------------
 struct ldpc_flow_ws {
-    size_t cap[4] = {0, 0, 0, 0};
-    void *buf[4] = {nullptr, nullptr, nullptr, nullptr};
-    void *ctl = nullptr, *sim = nullptr;  // sim: the simulation's state and its slots' frames
+    int frames = 0;                       // that the buffers serve
+    size_t cap[5] = {0, 0, 0, 0, 0};
+    void *buf[5] = {nullptr, nullptr, nullptr, nullptr, nullptr};  // as FlowMem's
     int log_cap = 0;
+    void *sim = nullptr;                  // the simulation's state and its slots' frames
     int *err = nullptr;                   // pinned, device-mapped
     unsigned long long *host = nullptr;   // pinned copy of the simulation's counters
 };
@@ -300,15 +301,16 @@ namespace ldpc {
 void flow_free(ldpc_flow_ws *w) {
     if (!w) return;
     for (void *b : w->buf) cudaFree(b);
-    cudaFree(w->ctl);
     cudaFree(w->sim);
     if (w->host) cudaFreeHost(w->host);
     if (w->err) cudaFreeHost(w->err);
     delete w;
 }
 
-// buffers for W slots
-static ldpc_status flow_ensure(ldpc_code c, int msg, int algo, bool post, int W, bool sim) {
+// buffers for a decode of `frames` frames, or a simulation on as many frame slots, by every rule and
+// message type, with posteriors or without: they are freed for larger ones by a call on more frames only
+// (as those of the launches, qc_ensure_workspace), so a captured call stays good while others decode
+static ldpc_status flow_ensure(ldpc_code c, int frames, bool sim) {
     auto fail = [&](size_t bytes) {
         cudaGetLastError();
         set_error("device allocation of the decoder's workspace (%zu bytes) failed", bytes);
@@ -319,17 +321,6 @@ static ldpc_status flow_ensure(ldpc_code c, int msg, int algo, bool post, int W,
         if (!c->flow) return fail(0);
     }
     ldpc_flow_ws &w = *c->flow;
-    const int log_cap = std::min(log_entries(W, flow_blocks()), kMaxLog);
-    if (log_cap > w.log_cap) {
-        if (w.ctl) LDPC_CUDA_TRY(cudaDeviceSynchronize());
-        cudaFree(w.ctl);
-        w.log_cap = 0;
-        if (cudaMalloc(&w.ctl, flow_ctl_bytes(kMaxSlots, log_cap)) != cudaSuccess) {
-            w.ctl = nullptr;
-            return fail(flow_ctl_bytes(kMaxSlots, log_cap));
-        }
-        w.log_cap = log_cap;
-    }
     if (!w.err) {
         if (cudaHostAlloc((void **)&w.err, 64, cudaHostAllocMapped) != cudaSuccess) {
             w.err = nullptr;
@@ -348,23 +339,39 @@ static ldpc_status flow_ensure(ldpc_code c, int msg, int algo, bool post, int W,
         w.host = nullptr;
         return fail(64);
     }
-    size_t b[4];
-    flow_slot_bytes(c->d, msg, algo, post, b);
+    if (frames <= w.frames) return LDPC_OK;
+    const long long cap = std::min(((long long)frames + 127) / 128 * 128, (long long)INT32_MAX);
+    size_t need[5] = {0, 0, 0, 0, 0};
+    int most = 1;
+    for (int form = 0; form < 6; ++form) {
+        static const int msgs[3] = {LDPC_MSG_F32, LDPC_MSG_F16, LDPC_MSG_I8};
+        const int msg = msgs[form / 2], algo = msg == LDPC_MSG_I8 ? LDPC_ALGO_MS : LDPC_ALGO_SP;
+        const bool post = form % 2 != 0;
+        const int wd = 32 * lanes_per_word(msg), W = flow_slots(c->d, msg, algo, post, (int)((cap + wd - 1) / wd));
+        size_t b[4];
+        flow_slot_bytes(c->d, msg, algo, post, b);
+        for (int i = 0; i < 4; ++i) need[i] = std::max(need[i], b[i] * W);
+        most = std::max(most, W);
+    }
+    const int log_cap = std::min(log_entries(most, flow_blocks()), kMaxLog);
+    need[4] = flow_ctl_bytes(kMaxSlots, log_cap);
     bool synced = false;
-    for (int i = 0; i < 4; ++i) {
-        const size_t need = b[i] * W;
-        if (need <= w.cap[i]) continue;
+    for (int i = 0; i < 5; ++i) {
+        if (need[i] <= w.cap[i]) continue;
         if (!synced) LDPC_CUDA_TRY(cudaDeviceSynchronize());
         synced = true;
         cudaFree(w.buf[i]);
         w.buf[i] = nullptr;
         w.cap[i] = 0;
-        if (cudaMalloc(&w.buf[i], need) != cudaSuccess) {
+        if (cudaMalloc(&w.buf[i], need[i]) != cudaSuccess) {
             w.buf[i] = nullptr;
-            return fail(need);
+            w.frames = 0;
+            return fail(need[i]);
         }
-        w.cap[i] = need;
+        w.cap[i] = need[i];
     }
+    w.log_cap = log_cap;
+    w.frames = (int)cap;
     return LDPC_OK;
 }
 
@@ -372,10 +379,10 @@ ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldp
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
     const int V = lanes_per_word(o.msg);
     const int W = flow_slots(c->d, o.msg, o.algo, post != nullptr, (gamma + 32 * V - 1) / (32 * V));
-    const ldpc_status e = flow_ensure(c, o.msg, o.algo, post != nullptr, W, false);
+    const ldpc_status e = flow_ensure(c, gamma, false);
     if (e != LDPC_OK) return e;
     const ldpc_flow_ws &w = *c->flow;
-    FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.log_cap, w.err};
+    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err};
     return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
 }
 
@@ -383,10 +390,10 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
                           const ldpc_decode_opts &o, unsigned long long *h, cudaStream_t s, const StreamIO *io) {
     const int V = lanes_per_word(o.msg);
     const int W = flow_slots(c->d, o.msg, o.algo, false, (slots + 32 * V - 1) / (32 * V));
-    ldpc_status e = flow_ensure(c, o.msg, o.algo, false, W, true);
+    ldpc_status e = flow_ensure(c, slots, true);
     if (e != LDPC_OK) return e;
     ldpc_flow_ws &w = *c->flow;
-    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.ctl, W, w.log_cap, w.err};
+    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err};
     std::memset(h, 0, 8 * sizeof(*h));
     constexpr int64_t kMost = (int64_t)1 << 20;  // frames a launch, so that none runs for minutes
     for (int64_t at = 0; at < max_frames; at += kMost) {

@@ -71,6 +71,15 @@ void fake_reset() {
     g_device = g_clusters = g_capturing = g_give_up = g_refused = 0;
     g_last = cudaSuccess;
 }
+void *fake_alloc(long long n) {  // device memory of the test's own
+    void *p = calloc(n ? n : 1, 1);
+    g_mem[(char *)p] = {(size_t)n, cudaMemoryTypeDevice};
+    return p;
+}
+void fake_free(void *p) {
+    g_mem.erase((char *)p);
+    free(p);
+}
 void fake_budget(long long bytes) { g_budget = bytes; }
 void fake_device(int dev) { g_device = dev; }
 void fake_clusters(int n) { g_clusters = n; }

@@ -31,6 +31,8 @@ class FakeDevice:
             f.restype, f.argtypes = res, args
         self.c.fake_launch_name.restype = ctypes.c_char_p
         self.c.fake_pinned_bytes.restype = ctypes.c_longlong
+        self.c.fake_alloc.restype, self.c.fake_alloc.argtypes = P, [ctypes.c_longlong]
+        self.c.fake_free.argtypes = [P]
         self.c.fake_budget.argtypes = [ctypes.c_longlong]
         self.keep = []
 
@@ -47,13 +49,16 @@ class FakeDevice:
         return h
 
     def device(self, nbytes):
-        p = P()
-        assert self.c.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(nbytes)) == 0
-        return p
+        return P(self.c.fake_alloc(nbytes))
+
+    def calls(self, name):
+        return self.c.fake_calls(name.encode())
 
     def decode(self, code, N, gamma, *, noalloc=False, post=False, host_out=False, **opts):
         """ldpc_decode (or _noalloc) on device buffers, the decisions to the host with host_out; the status"""
         o = pkg.default_opts(**opts)
+        prm = self.device(8 * 256 * o.max_iter) if o.algo == pkg.ALGO_NOMS else None
+        o.noms_params = prm
         llr = self.device(4 * gamma * N)
         d_post = self.device(4 * gamma * N) if post else None
         if host_out:
@@ -64,9 +69,9 @@ class FakeDevice:
             hard = self.device(gamma * N)
         f = self.c.ldpc_decode_noalloc if noalloc else self.c.ldpc_decode
         st = f(code, llr, gamma, ctypes.byref(o), d_post, hard, None, None, None)
-        for x in (llr, d_post, None if host_out else hard):
+        for x in (prm, llr, d_post, None if host_out else hard):
             if x is not None:
-                self.c.cudaFree(x)
+                self.c.fake_free(x)
         return st
 
     def sim(self, code, frames, slots, target=1 << 60, **opts):

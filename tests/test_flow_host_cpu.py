@@ -83,3 +83,26 @@ def test_log_entry_read_in_two_parts(dev, length):
         assert dev.c.fake_entry_is(before, n, n) == ahead and dev.c.fake_entry_is(n, before, n) == ahead
         assert dev.c.fake_entry_is(after, after, n) == past and dev.c.fake_entry_is(n, after, n) == past
         assert dev.c.fake_entry_is(after, n, n) == ahead  # read again: n has been overwritten
+
+
+@pytest.mark.parametrize("J,L,p", [(4, 24, 211), (4, 24, 765), (8, 32, 200)])
+def test_buffers_are_kept_while_batches_do_not_grow(dev, J, L, p):
+    """Once a batch has been decoded, no decode of as many frames or fewer and no simulation on as many slots
+    frees a buffer (one that a captured graph of the first call holds) or needs memory that the first did not."""
+    code = dev.code(J, L, p)
+    N, frames = L * p, 700
+    assert dev.decode(code, N, frames, max_iter=30) == 0
+    assert len(dev.flows()) == 1
+    had = dev.calls("cudaMalloc")
+    for algo, msg in ((0, 0), (0, 1), (1, 2), (2, 0), (2, 1)):
+        for post in (False, True):
+            for early in (0, 1):
+                for n in (frames, 701 - 128, 33):
+                    assert dev.decode(code, N, n, post=post, algo=algo, msg=msg, early_stop=early, max_iter=30) == 0
+    flows = dev.flows()
+    assert len(flows) > 40 and dev.calls("cudaFree") == 0
+    # (the calls that go by launches have a workspace of their own: eight buffers)
+    assert dev.calls("cudaMalloc") <= had + 8
+    assert dev.sim(code, 2000, 700, early_stop=1) == 0  # and the simulation its state: one
+    assert dev.calls("cudaMalloc") <= had + 9 and dev.calls("cudaFree") == 0
+    dev.c.ldpc_code_destroy(code)
