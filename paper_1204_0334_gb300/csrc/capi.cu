@@ -351,6 +351,46 @@ static int stream_slots(const ldpc_code c, int gamma, const ldpc_decode_opts &o,
     return gamma >= 2 * slots ? slots : 0;
 }
 
+// a launch per pass, on the code's workspace
+static ldpc_status launches_decode(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
+                                   uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+    ldpc_status st = qc_ensure_workspace(c, (size_t)gamma);
+    if (st != LDPC_OK) return st;
+    st = qc_pack_llr(c, llr, gamma, o, s);
+    if (st != LDPC_OK) return st;
+    st = qc_decode_device(c, gamma, o, post != nullptr, s);
+    if (st != LDPC_OK) return st;
+    return qc_unpack_outputs(c, gamma, o, post, hard, iters, ok, s);
+}
+
+// A decode on device buffers by the form that is faster: on chip, as one launch, or by launches.  All give the
+// same results, so a call on no more frames than an earlier one needs no memory that cannot be had: where
+// the faster form's workspace is not there and cannot be made (under capture, or out of memory), another
+// form is taken whose workspace is.
+static ldpc_status decode_frames(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
+                                 uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
+    if (c->sparse) return launches_decode(c, llr, gamma, o, post, hard, iters, ok, s);
+    bool on_chip = false;
+    ldpc_status st = chip_decode(c->d, llr, gamma, o, post, hard, iters, ok, s, &on_chip);
+    if (st != LDPC_OK || on_chip) return st;
+    const bool flow_here = flow_ready(c, gamma), launches_here = (size_t)gamma <= c->ws.gamma_cap;
+    const bool flow = flow_pays(c->d, gamma, o), here = flow ? flow_here : launches_here;
+    cudaStreamCaptureStatus capture = cudaStreamCaptureStatusNone;
+    if (!here) LDPC_CUDA_TRY(cudaStreamIsCapturing(s, &capture));
+    if (here || capture == cudaStreamCaptureStatusNone) {
+        st = flow ? flow_decode_code(c, llr, gamma, o, post, hard, iters, ok, s)
+                  : launches_decode(c, llr, gamma, o, post, hard, iters, ok, s);
+        if (here || st != LDPC_ENOMEM) return st;
+    }
+    if (flow && launches_here) return launches_decode(c, llr, gamma, o, post, hard, iters, ok, s);
+    if (!flow && flow_here) return flow_decode_code(c, llr, gamma, o, post, hard, iters, ok, s);
+    const ldpc_status any = chip_decode(c->d, llr, gamma, o, post, hard, iters, ok, s, &on_chip, true);
+    if (any != LDPC_OK || on_chip) return any;
+    if (capture == cudaStreamCaptureStatusNone) return st;
+    return flow ? flow_decode_code(c, llr, gamma, o, post, hard, iters, ok, s)
+                : launches_decode(c, llr, gamma, o, post, hard, iters, ok, s);
+}
+
 ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc_decode_opts *opts, float *post,
                         uint8_t *hard, int32_t *iters, int32_t *ok, void *stream) {
     if (!c || !llr || gamma < 1) {
@@ -391,24 +431,8 @@ ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc
     uint8_t *d_hard = hard && pointer_kind(hard) == 1 ? w.stage_hard : hard;
     int32_t *d_iters = iters && pointer_kind(iters) == 1 ? w.stage_i32 : iters;
     int32_t *d_ok = ok && pointer_kind(ok) == 1 ? w.stage_i32 + w.stage_cap : ok;
-    bool on_chip = false;
-    if (!c->sparse) {
-        st = chip_decode(c->d, src, gamma, o, d_post, d_hard, d_iters, d_ok, s, &on_chip);
-        if (st != LDPC_OK) return st;
-    }
-    if (!on_chip && !c->sparse && flow_pays(c->d, gamma, o)) {
-        st = flow_decode_code(c, src, gamma, o, d_post, d_hard, d_iters, d_ok, s);
-        if (st != LDPC_OK) return st;
-    } else if (!on_chip) {
-        st = qc_ensure_workspace(c, (size_t)gamma);
-        if (st != LDPC_OK) return st;
-        st = qc_pack_llr(c, src, gamma, o, s);
-        if (st != LDPC_OK) return st;
-        st = qc_decode_device(c, gamma, o, post != nullptr, s);
-        if (st != LDPC_OK) return st;
-        st = qc_unpack_outputs(c, gamma, o, d_post, d_hard, d_iters, d_ok, s);
-        if (st != LDPC_OK) return st;
-    }
+    st = decode_frames(c, src, gamma, o, d_post, d_hard, d_iters, d_ok, s);
+    if (st != LDPC_OK) return st;
     if (d_post != post) LDPC_CUDA_TRY(cudaMemcpyAsync(post, d_post, NB * 4, cudaMemcpyDeviceToHost, s));
     if (d_hard != hard) LDPC_CUDA_TRY(cudaMemcpyAsync(hard, d_hard, NB, cudaMemcpyDeviceToHost, s));
     if (d_iters != iters) LDPC_CUDA_TRY(cudaMemcpyAsync(iters, d_iters, (size_t)gamma * 4, cudaMemcpyDeviceToHost, s));

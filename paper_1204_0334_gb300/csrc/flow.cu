@@ -375,6 +375,8 @@ static ldpc_status flow_ensure(ldpc_code c, int frames, bool sim) {
     return LDPC_OK;
 }
 
+bool flow_ready(const ldpc_code c, int gamma) { return c->flow && gamma <= c->flow->frames; }
+
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s) {
     const int V = lanes_per_word(o.msg);

@@ -55,7 +55,7 @@ int pick(const void *kernel, const Code &c, int V, bool ms, const ChipArgs &a, i
     for (int i = 0; i < c.J * c.L; ++i) E += c.sh[i] >= 0 ? c.p : 0;
     for (int C = 16; C >= 1; C /= 2) {
         const int NC = (c.N + C - 1) / C;
-        if (bytes(c, V, ms, a.want_post, NC) > kChipMost || E > C * most_lines(c, V, P, a.early)) return 0;  // fewer blocks hold less
+        if (bytes(c, V, ms, a.want_post, NC) > kChipMost || (!a.any && E > C * most_lines(c, V, P, a.early))) return 0;  // fewer blocks hold less
         if ((C - 1) * NC >= c.N) continue;  // a block would have no variable
         const auto key = std::make_pair(kernel, C);
         auto f = active.find(key);
@@ -90,7 +90,7 @@ using namespace flow;
 
 // Takes a decode whose packages all fit on the chip at once; *taken says whether it did.
 ldpc_status chip_decode(const QcDesc &d, const float *llr, int gamma, const ldpc_decode_opts &o, float *post, uint8_t *hard,
-                        int32_t *iters, int32_t *ok, cudaStream_t s, bool *taken) {
+                        int32_t *iters, int32_t *ok, cudaStream_t s, bool *taken, bool any) {
     const int V = lanes_per_word(o.msg), P = (gamma + 32 * V - 1) / (32 * V);
     *taken = false;
     if (P > 152 || d.E > 16 * 800) return LDPC_OK;
@@ -104,6 +104,7 @@ ldpc_status chip_decode(const QcDesc &d, const float *llr, int gamma, const ldpc
     c.nparams = o.algo == LDPC_ALGO_NOMS ? o.noms_params : nullptr;
     chip::ChipArgs a;
     std::memset(&a, 0, sizeof(a));
+    a.any = any;
     a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post != nullptr;
     a.clip = o.clip, a.qscale = ldexpf(1.0f, o.frac_bits), a.lsb = ldexpf(1.0f, -o.frac_bits);
     if (o.algo == LDPC_ALGO_MS) return chip::run_ms(c, a, P, s, taken);

@@ -195,9 +195,12 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
 
-// the on-chip decoder of short codes (flow_chip.cu)
+// whether that workspace serves gamma frames as it is
+bool flow_ready(const ldpc_code c, int gamma);
+
+// the on-chip decoder of short codes (flow_chip.cu); any: also where another form is faster
 ldpc_status chip_decode(const QcDesc &d, const float *llr, int gamma, const ldpc_decode_opts &o, float *post, uint8_t *hard,
-                        int32_t *iters, int32_t *ok, cudaStream_t s, bool *taken);
+                        int32_t *iters, int32_t *ok, cudaStream_t s, bool *taken, bool any = false);
 
 namespace chip {
 
@@ -210,6 +213,7 @@ struct ChipArgs {
     int C, NC;       // blocks of a cluster, variables of a block
     FastDiv divNC;
     int max_iter, early, want_post;
+    int any;         // taken also where another form is faster
     float clip, qscale, lsb;
 };
 size_t bytes(const flow::Code &c, int V, bool ms, bool post, int NC);

@@ -464,7 +464,10 @@ ldpc_status qc_ber_sim_refill(ldpc_code c, double sigma, uint64_t seed, uint64_t
     // one launch where the frames' results do not depend on how many are in flight: a frame-error target
     // that cannot be met (or a caller's batch), all-zero codewords, one rule for every frame
     if (o.algo != LDPC_ALGO_NOMS && flow_sim_pays(c->d, gamma, o) && (io || (o.codewords == LDPC_CODEWORDS_ZERO && target > max_frames)))
-        return flow_sim_code(c, sigma, seed, first_frame, max_frames, gamma, o, h, s, io);
+    {
+        const ldpc_status e = flow_sim_code(c, sigma, seed, first_frame, max_frames, gamma, o, h, s, io);
+        if (e != LDPC_ENOMEM || (size_t)gamma > c->ws.gamma_cap) return e;
+    }
     const int V = lanes_per_word(o.msg), W = 32 * V;
     const int P = (gamma + W - 1) / W;
     const size_t slots = (size_t)P * W;

@@ -31,7 +31,7 @@ std::map<std::string, int> g_calls;
 std::map<std::pair<int, const void *>, int> g_smem;  // (device, kernel) -> shared memory it may have
 ldpc::flow::Start g_start;
 long long g_budget = -1;  // bytes of device memory still to be had (-1: any)
-int g_device = 0, g_clusters = 0, g_capturing = 0, g_give_up = 0, g_refused = 0;
+int g_device = 0, g_capturing = 0, g_give_up = 0, g_refused = 0;
 cudaError_t g_last = cudaSuccess;
 struct {
     dim3 grid, block;
@@ -68,7 +68,7 @@ void fake_reset() {
     g_launches.clear();
     g_calls.clear();
     g_budget = -1;
-    g_device = g_clusters = g_capturing = g_give_up = g_refused = 0;
+    g_device = g_capturing = g_give_up = g_refused = 0;
     g_last = cudaSuccess;
 }
 void *fake_alloc(long long n) {  // device memory of the test's own
@@ -82,7 +82,6 @@ void fake_free(void *p) {
 }
 void fake_budget(long long bytes) { g_budget = bytes; }
 void fake_device(int dev) { g_device = dev; }
-void fake_clusters(int n) { g_clusters = n; }
 void fake_capturing(int on) { g_capturing = on; }
 void fake_give_up(int code) { g_give_up = code; }  // the next flow launch gives up a wait
 int fake_refused() { return g_refused; }
@@ -232,8 +231,8 @@ cudaError_t cudaOccupancyMaxActiveBlocksPerMultiprocessorWithFlags(int *n, const
     *n = 1;
     return cudaSuccess;
 }
-cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *) {
-    *n = g_clusters;
+cudaError_t cudaOccupancyMaxActiveClusters(int *n, const void *, const cudaLaunchConfig_t *c) {
+    *n = 152 / (int)c->gridDim.x;  // one cluster asked about: a block an SM
     return cudaSuccess;
 }
 cudaError_t cudaGetLastError() {

@@ -106,3 +106,34 @@ def test_buffers_are_kept_while_batches_do_not_grow(dev, J, L, p):
     assert dev.sim(code, 2000, 700, early_stop=1) == 0  # and the simulation its state: one
     assert dev.calls("cudaMalloc") <= had + 9 and dev.calls("cudaFree") == 0
     dev.c.ldpc_code_destroy(code)
+
+
+def form(dev):
+    """how the last decode ran"""
+    last = dev.names()[-1]
+    return "chip" if "chip_kernel" in last else "flow" if "tile_kernel" in last else "launches"
+
+
+# a batch decoded first, then one of no more frames that by itself takes another form
+OTHERS = [((4, 24, 765), dict(gamma=2048, early_stop=1), dict(gamma=32), "flow", "launches"),
+          ((4, 24, 211), dict(gamma=96), dict(gamma=33, early_stop=1), "launches", "flow"),
+          ((4, 12, 200), dict(gamma=512, algo=1, msg=2), dict(gamma=128, algo=1, msg=2), "chip", "launches")]
+
+
+@pytest.mark.parametrize("shape,first,then,before,alone", OTHERS)
+def test_smaller_batch_without_new_memory(dev, shape, first, then, before, alone):
+    """Under capture, and where no memory is left, a batch of no more frames than an earlier one is decoded
+    by the form whose workspace is there."""
+    N = shape[1] * shape[2]
+    for how in ("alone", "capture", "no memory"):
+        code = dev.code(*shape)
+        if how != "alone":
+            assert dev.decode(code, N, max_iter=20, **first) == 0 and form(dev) == before
+        dev.c.fake_capturing(how == "capture")
+        if how == "no memory":
+            dev.c.fake_budget(0)
+        st = dev.decode(code, N, max_iter=20, **then)
+        dev.c.fake_capturing(0)
+        dev.c.fake_budget(-1)
+        assert st == 0 and form(dev) == (alone if how == "alone" else before), how
+        dev.c.ldpc_code_destroy(code)

@@ -53,3 +53,31 @@ def test_decode_of_more_packages_than_slots(pkg):
         assert n == 1  # on chip
         for a, b in zip(whole, part):
             assert torch.equal(a[f:f + 3000], b)
+
+
+def test_captured_decodes(pkg):
+    """A decode captured after a larger batch that ran in another form, and one replayed after decodes of the
+    same frames with other messages and outputs have run on the object."""
+    shifts = synth.qc_shifts(4, 24, 765, seed=2)
+    code, other = pkg.QCCode(shifts, 765), pkg.QCCode(shifts, 765)
+    mu = code.channel(3.0, 5, 0, 600)
+    opts = pkg.default_opts(max_iter=6)
+
+    def outputs(n):
+        return (torch.empty((n, code.N), device="cuda"), torch.empty((n, code.N), dtype=torch.uint8, device="cuda"),
+                torch.empty(n, dtype=torch.int32, device="cuda"), torch.empty(n, dtype=torch.int32, device="cuda"))
+
+    code.decode(mu, max_iter=6, early_stop=True)
+    small, whole = outputs(32), outputs(600)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        pkg.ldpc_decode(code.handle, mu[:32], opts, *small)
+        pkg.ldpc_decode(code.handle, mu, opts, None, *whole[1:])
+    for msg, algo in ((pkg.MSG_F16, pkg.ALGO_SP), (pkg.MSG_I8, pkg.ALGO_MS)):
+        code.decode(mu, max_iter=6, msg=msg, algo=algo)
+    graph.replay()
+    torch.cuda.synchronize()
+    for a, b in zip(small, other.decode(mu[:32], max_iter=6)):
+        assert torch.equal(a, b)
+    for a, b in zip(whole[1:], other.decode(mu, max_iter=6)[1:]):
+        assert torch.equal(a, b)
