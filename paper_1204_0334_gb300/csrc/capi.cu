@@ -399,6 +399,8 @@ ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc
     }
     ldpc_status st = check_opts(c, opts);
     if (st != LDPC_OK) return st;
+    st = flow_check(c, "an earlier decode of this object");
+    if (st != LDPC_OK) return st;
     const ldpc_decode_opts &o = *opts;
     cudaStream_t s = (cudaStream_t)stream;
     if (const int slots = stream_slots(c, gamma, o, post)) {
@@ -486,6 +488,8 @@ ldpc_status ldpc_tune_slots(ldpc_code c, double ebn0_db, uint64_t seed, const ld
         set_error("design rate K/N = %g is not positive", c->rate);
         return LDPC_EINVAL;
     }
+    st = flow_check(c, "an earlier decode of this object");
+    if (st != LDPC_OK) return st;
     const ldpc_decode_opts &o = *opts;
     cudaStream_t s = (cudaStream_t)stream;
     const double sigma = channel_sigma(c, ebn0_db);
@@ -540,6 +544,8 @@ ldpc_status ldpc_ber_sim(ldpc_code c, double ebn0_db, uint64_t seed, uint64_t fi
         return LDPC_EUNSUPPORTED;
     }
     ldpc_status st = check_opts(c, opts);
+    if (st != LDPC_OK) return st;
+    st = flow_check(c, "an earlier decode of this object");
     if (st != LDPC_OK) return st;
     const ldpc_decode_opts &o = *opts;
     cudaStream_t s = (cudaStream_t)stream;

@@ -221,11 +221,6 @@ bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o) {
 static ldpc_status prepare(const QcDesc &d, const FlowMem &m, const ldpc_decode_opts &o, int W, bool post, Start &st, Args &a,
                            uint32_t *tiles) {
     const int V = lanes_per_word(o.msg), FV = o.algo == LDPC_ALGO_MS ? 1 : V;
-    if (m.err && *(volatile int *)m.err) {
-        set_error("an earlier decode of this object gave up a device-side wait (code %d)", *m.err);
-        *m.err = 0;
-        return LDPC_ETIMEOUT;
-    }
     std::memset(&st, 0, sizeof(st));
     *tiles = fill_code(d, FV, st.code);
     if (*tiles >= (1u << kLogTiles) || o.max_iter >= (1 << kLogIt)) {
@@ -375,6 +370,16 @@ static ldpc_status flow_ensure(ldpc_code c, int frames, bool sim) {
     return LDPC_OK;
 }
 
+ldpc_status flow_gave_up(int *err, const char *what) {
+    const int e = err ? *(volatile int *)err : 0;
+    if (!e) return LDPC_OK;
+    *err = 0;
+    set_error("%s gave up a device-side wait (code %d)", what, e);
+    return LDPC_ETIMEOUT;
+}
+
+ldpc_status flow_check(const ldpc_code c, const char *what) { return flow_gave_up(c->flow ? c->flow->err : nullptr, what); }
+
 bool flow_ready(const ldpc_code c, int gamma) { return c->flow && gamma <= c->flow->frames; }
 
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
@@ -424,11 +429,8 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
         if (e != LDPC_OK) return e;
         LDPC_CUDA_TRY(cudaMemcpyAsync(w.host, a.sim->counters, 64, cudaMemcpyDeviceToHost, s));
         LDPC_CUDA_TRY(cudaStreamSynchronize(s));
-        if (*(volatile int *)w.err) {
-            set_error("the simulation gave up a device-side wait (code %d)", *w.err);
-            *w.err = 0;
-            return LDPC_ETIMEOUT;
-        }
+        e = flow_check(c, "the simulation");
+        if (e != LDPC_OK) return e;
         for (int i = 0; i < 8; ++i) h[i] += w.host[i];
     }
     return LDPC_OK;

@@ -195,6 +195,9 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
 
+// LDPC_ETIMEOUT, once, if a launch has set its word (no wait: launches that are done by now)
+ldpc_status flow_gave_up(int *err, const char *what);
+ldpc_status flow_check(const ldpc_code c, const char *what);
 // whether that workspace serves gamma frames as it is
 bool flow_ready(const ldpc_code c, int gamma);
 

@@ -124,6 +124,8 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
     int *err = nullptr;
     st = noalloc_base(&base_v, &ctl, &err);
     if (st != LDPC_OK) return st;
+    st = flow_gave_up(err, "an earlier decode in the fixed scratch");
+    if (st != LDPC_OK) return st;
     noalloc_need(c->d, cap, off);
     unsigned char *base = (unsigned char *)base_v;
     cudaStream_t s = (cudaStream_t)stream;

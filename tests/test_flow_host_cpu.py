@@ -137,3 +137,29 @@ def test_smaller_batch_without_new_memory(dev, shape, first, then, before, alone
         dev.c.fake_budget(-1)
         assert st == 0 and form(dev) == (alone if how == "alone" else before), how
         dev.c.ldpc_code_destroy(code)
+
+
+OK, ETIMEOUT = 0, 4
+
+
+def test_a_wait_given_up_is_told_by_the_next_call(dev):
+    """A device-side wait that gave up is told by the next call on the object, whichever way that runs, and
+    by no other and no later one."""
+    code, other = dev.code(4, 24, 211), dev.code(4, 24, 211)
+    N = 24 * 211
+    big, few = dict(gamma=4096, max_iter=30), dict(gamma=32, max_iter=30)
+    for then in (lambda: dev.decode(code, N, **big), lambda: dev.decode(code, N, **few),
+                 lambda: dev.sim(code, 500, 64, early_stop=1), lambda: dev.sim(code, 500, 64, target=100),
+                 lambda: dev.decode(code, N, gamma=8192, early_stop=1, max_iter=30)):
+        assert then() == OK  # each of them runs by itself
+        dev.c.fake_give_up(1)
+        assert dev.decode(code, N, **big) == OK and form(dev) == "flow"
+        n = len(dev.names())
+        assert dev.decode(other, N, **big) == OK
+        assert then() == ETIMEOUT
+        assert then() == OK and len(dev.names()) > n
+    dev.c.fake_give_up(2)  # a call that waits tells of its own
+    assert dev.sim(code, 500, 64, early_stop=1) == ETIMEOUT
+    assert dev.decode(code, N, **big) == OK
+    dev.c.ldpc_code_destroy(code)
+    dev.c.ldpc_code_destroy(other)
