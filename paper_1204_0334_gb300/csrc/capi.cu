@@ -337,6 +337,14 @@ static void *mapped_ptr(const void *p) {
     return nullptr;
 }
 
+static bool pageable(const void *p) {
+    if (!p) return false;
+    cudaPointerAttributes a;
+    if (cudaPointerGetAttributes(&a, p) == cudaSuccess) return a.type == cudaMemoryTypeUnregistered;
+    cudaGetLastError();
+    return true;
+}
+
 // Slot count of the streaming decode, or 0 when ldpc_decode keeps its batch path: the stream
 // gives every frame exactly the batch path's iterations and decisions (QC codes, sum-product
 // with FP32 messages or integer min-sum, early stop -- without it a stream has nothing to
@@ -439,6 +447,8 @@ ldpc_status ldpc_decode(ldpc_code c, const float *llr, int32_t gamma, const ldpc
     if (d_hard != hard) LDPC_CUDA_TRY(cudaMemcpyAsync(hard, d_hard, NB, cudaMemcpyDeviceToHost, s));
     if (d_iters != iters) LDPC_CUDA_TRY(cudaMemcpyAsync(iters, d_iters, (size_t)gamma * 4, cudaMemcpyDeviceToHost, s));
     if (d_ok != ok) LDPC_CUDA_TRY(cudaMemcpyAsync(ok, d_ok, (size_t)gamma * 4, cudaMemcpyDeviceToHost, s));
+    // a copy to pageable memory returns when it is done, and with it the decode
+    if (pageable(post) || pageable(hard) || pageable(iters) || pageable(ok)) return flow_check(c, "the decode");
     return LDPC_OK;
 }
 

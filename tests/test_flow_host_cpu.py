@@ -163,3 +163,14 @@ def test_a_wait_given_up_is_told_by_the_next_call(dev):
     assert dev.decode(code, N, **big) == OK
     dev.c.ldpc_code_destroy(code)
     dev.c.ldpc_code_destroy(other)
+
+
+def test_a_wait_given_up_with_pageable_outputs(dev):
+    """Outputs in pageable host memory are there when the call returns: it tells of its own time-out."""
+    code = dev.code(4, 24, 211)
+    big = dict(gamma=4096, max_iter=30)
+    dev.c.fake_give_up(3)
+    assert dev.decode(code, 24 * 211, host_out=True, **big) == ETIMEOUT
+    assert dev.decode(code, 24 * 211, host_out=True, **big) == OK
+    assert dev.decode(code, 24 * 211, **big) == OK
+    dev.c.ldpc_code_destroy(code)
