@@ -136,8 +136,8 @@ ldpc_status ldpc_code_dims(ldpc_code code, int64_t *N, int64_t *M, int64_t *E, i
  * A batch of a QC code runs as one launch where that is faster; every form gives
  * the same results.  If a wait on the device gives up (it has a limit), a form that
  * does not wait reports LDPC_ETIMEOUT on the next ldpc_decode, ldpc_ber_sim or
- * ldpc_tune_slots on the code, which is not carried out (ldpc_decode_noalloc: its next
- * call).  A call whose outputs are in pageable host memory has waited for them and
+ * ldpc_tune_slots on the code, which is not carried out (ldpc_decode_noalloc: on its
+ * next call on the code).  A call whose outputs are in pageable host memory has waited for them and
  * reports its own.
  * Errors: LDPC_EINVAL (null code/llr, gamma < 1, bad opts), LDPC_EUNSUPPORTED
  * (algo/msg pair not built), LDPC_ENOMEM, LDPC_ECUDA, LDPC_ETIMEOUT.

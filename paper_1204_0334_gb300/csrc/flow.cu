@@ -243,6 +243,7 @@ static ldpc_status prepare(const QcDesc &d, const FlowMem &m, const ldpc_decode_
     a.max_iter = o.max_iter, a.early = o.early_stop != 0, a.want_post = post;
     a.clip = o.clip, a.qscale = ldexpf(1.0f, o.frac_bits), a.lsb = ldexpf(1.0f, -o.frac_bits);
     a.err = m.err;
+    a.err_tag = m.err_tag;
     return LDPC_OK;
 }
 
@@ -370,15 +371,15 @@ static ldpc_status flow_ensure(ldpc_code c, int frames, bool sim) {
     return LDPC_OK;
 }
 
-ldpc_status flow_gave_up(int *err, const char *what) {
+ldpc_status flow_gave_up(int *err, int tag, const char *what) {
     const int e = err ? *(volatile int *)err : 0;
-    if (!e) return LDPC_OK;
+    if (!e || (e & ~7) != tag) return LDPC_OK;
     *err = 0;
-    set_error("%s gave up a device-side wait (code %d)", what, e);
+    set_error("%s gave up a device-side wait (code %d)", what, e & 7);
     return LDPC_ETIMEOUT;
 }
 
-ldpc_status flow_check(const ldpc_code c, const char *what) { return flow_gave_up(c->flow ? c->flow->err : nullptr, what); }
+ldpc_status flow_check(const ldpc_code c, const char *what) { return flow_gave_up(c->flow ? c->flow->err : nullptr, 0, what); }
 
 bool flow_ready(const ldpc_code c, int gamma) { return c->flow && gamma <= c->flow->frames; }
 
@@ -389,7 +390,7 @@ ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldp
     const ldpc_status e = flow_ensure(c, gamma, false);
     if (e != LDPC_OK) return e;
     const ldpc_flow_ws &w = *c->flow;
-    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err};
+    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err, 0};
     return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
 }
 
@@ -400,7 +401,7 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
     ldpc_status e = flow_ensure(c, slots, true);
     if (e != LDPC_OK) return e;
     ldpc_flow_ws &w = *c->flow;
-    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err};
+    const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err, 0};
     std::memset(h, 0, 8 * sizeof(*h));
     constexpr int64_t kMost = (int64_t)1 << 20;  // frames a launch, so that none runs for minutes
     for (int64_t at = 0; at < max_frames; at += kMost) {

@@ -738,7 +738,7 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
         if ((++tries & 15) == 0) {
             if (ld_int(&a.ctl->abort)) return false;
             if (tries > kLookLimit) {
-                if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = 1;
+                if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = a.err_tag | 1;
                 return false;
             }
         }
@@ -1008,7 +1008,7 @@ __device__ __forceinline__ void taking_warp(const Args &a, SM &sm, int lane) {
         uint32_t idx = 0u;  // taken while the stage empties
         bool on = take(a, lane, pl, idx);
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sm.empty[head]), ph))) {
-            if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = 3;
+            if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = a.err_tag | 3;
             on = false;
         }
         const uint32_t bar = smem_u32(&sm.full[head]);
@@ -1156,7 +1156,7 @@ template <typename C, int V, typename SM>
 __device__ __forceinline__ void retiring_warp(const Args &a, SM &sm, int st, int lane) {
     for (uint32_t ph = 0u;; ph ^= 1u) {
         if (!__all_sync(0xffffffffu, mbar_wait(smem_u32(&sm.used[st]), ph))) {
-            if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = 4;
+            if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = a.err_tag | 4;
             return;
         }
         const Desc &d = sm.desc[st];
@@ -1224,7 +1224,7 @@ __global__ void __launch_bounds__(kThreads, 1) tile_kernel(const Args a) {
     uint32_t ph = 0u;
     for (;;) {
         if (!mbar_wait(smem_u32(&sm.full[st]), ph)) {
-            if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = 2;
+            if (lane == 0) atomicExch(&a.ctl->abort, 1), *(volatile int *)a.err = a.err_tag | 2;
             return;
         }
         const Desc &d = sm.desc[st];

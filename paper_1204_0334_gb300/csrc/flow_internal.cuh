@@ -142,7 +142,8 @@ struct Args {
     float clip, qscale, lsb;
     Sim *sim;                  // refill mode, else NULL
     SimSlot *simslots;
-    int *err;                  // host word set when a wait ran out
+    int *err;                  // host word set when a wait ran out: which (1 to 4), beside err_tag
+    int err_tag;               // whose launch it is, where objects share a word (a multiple of 8)
 };
 
 struct Shape {
@@ -175,7 +176,7 @@ struct FlowMem {
     void *msg, *mu, *post, *hw;  // W slots each
     void *ctl;                   // flow_ctl_bytes()
     int W, log_cap;              // slots, entries of the phase log
-    int *err;
+    int *err, err_tag;
 };
 size_t flow_ctl_bytes(int W, int log_cap);
 // slots a decode of P packages keeps in work, and the bytes of one slot's buffers
@@ -195,8 +196,8 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
 ldpc_status flow_decode_code(ldpc_code c, const float *llr, int gamma, const ldpc_decode_opts &o, float *post,
                              uint8_t *hard, int32_t *iters, int32_t *ok, cudaStream_t s);
 
-// LDPC_ETIMEOUT, once, if a launch has set its word (no wait: launches that are done by now)
-ldpc_status flow_gave_up(int *err, const char *what);
+// LDPC_ETIMEOUT, once, if a launch with this tag has set its word (no wait: launches that are done by now)
+ldpc_status flow_gave_up(int *err, int tag, const char *what);
 ldpc_status flow_check(const ldpc_code c, const char *what);
 // whether that workspace serves gamma frames as it is
 bool flow_ready(const ldpc_code c, int gamma);

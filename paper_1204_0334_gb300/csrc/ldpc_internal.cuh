@@ -4,6 +4,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdint>
 #include <mutex>
 #include <string>
@@ -100,9 +101,16 @@ struct ldpc_code_s {
     std::mutex enc_mu;
     std::vector<int> h_rp, h_col;    // sparse code: H in compressed-row form (host copy)
     int device = 0;
+    uint32_t number = next_number();  // tells the objects of a process apart
     double rate = 0.0;   // design rate K/N
     int tuned_slots[3][3] = {};      // slot count picked by ldpc_tune_slots, per [algo][msg] (0 = not tuned)
     ldpc::DecodeWs ws;
+
+  private:
+    static uint32_t next_number() {
+        static std::atomic<uint32_t> last{0};
+        return ++last;
+    }
 };
 
 namespace ldpc {

@@ -40,7 +40,8 @@ namespace {
 constexpr int kMaxDevices = 64;
 std::mutex g_noalloc_mu;
 void *g_noalloc_ptr[kMaxDevices] = {}, *g_noalloc_ctl_ptr[kMaxDevices] = {};
-int *g_noalloc_err[kMaxDevices] = {};  // pinned host words the flow decoder reports to
+constexpr int kErrWords = 1024;
+int *g_noalloc_err[kMaxDevices] = {};  // pinned host words the flow decoder reports to, by the code's number
 
 // device addresses of the scratch arrays on the current device (looked up once per device)
 ldpc_status noalloc_base(void **out, void **ctl, int **err) {
@@ -57,9 +58,9 @@ ldpc_status noalloc_base(void **out, void **ctl, int **err) {
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_scratch)");
         e = cudaGetSymbolAddress(&g_noalloc_ctl_ptr[dev], g_noalloc_ctl);
         if (e != cudaSuccess) return cuda_fail(e, "cudaGetSymbolAddress(g_noalloc_ctl)");
-        e = cudaHostAlloc((void **)&g_noalloc_err[dev], 64, cudaHostAllocMapped);
+        e = cudaHostAlloc((void **)&g_noalloc_err[dev], kErrWords * sizeof(int), cudaHostAllocMapped);
         if (e != cudaSuccess) return cuda_fail(e, "cudaHostAlloc");
-        *g_noalloc_err[dev] = 0;
+        std::memset(g_noalloc_err[dev], 0, kErrWords * sizeof(int));
         g_noalloc_ptr[dev] = p;
     }
     *out = g_noalloc_ptr[dev];
@@ -124,7 +125,10 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
     int *err = nullptr;
     st = noalloc_base(&base_v, &ctl, &err);
     if (st != LDPC_OK) return st;
-    st = flow_gave_up(err, "an earlier decode in the fixed scratch");
+    // this code's word, and its number in it: another code may share the word, and is told for itself
+    const int tag = (int)(c->number % (INT32_MAX / 8)) * 8;
+    err += c->number % kErrWords;
+    st = flow_gave_up(err, tag, "an earlier decode of this object in the fixed scratch");
     if (st != LDPC_OK) return st;
     noalloc_need(c->d, cap, off);
     unsigned char *base = (unsigned char *)base_v;
@@ -142,7 +146,7 @@ ldpc_status ldpc_decode_noalloc(ldpc_code c, const float *llr, int32_t gamma, co
         flow_slot_bytes(c->d, o.msg, o.algo, post != nullptr, b);
         const int W = std::min((gamma + 32 * V - 1) / (32 * V), flow::kMaxSlots);
         for (int i = 0; i < 4; ++i) at[i] = x, x += b[i] * W;
-        const FlowMem m{base + at[0], base + at[1], base + at[2], base + at[3], ctl, W, flow::kMaxLog, err};
+        const FlowMem m{base + at[0], base + at[1], base + at[2], base + at[3], ctl, W, flow::kMaxLog, err, tag};
         return flow_decode(c->d, m, llr, gamma, o, post, hard, iters, ok, s);
     }
     // A private view of the code object whose workspace points into the scratch.  It

@@ -54,7 +54,7 @@ cudaError_t launch(const void *fn, dim3 grid, size_t smem, void **args) {
     if (l.name.find("tile_kernel") != std::string::npos && l.name.find("flow") != std::string::npos) {
         l.flow = *(const ldpc::flow::Args *)args[0];
         l.start = g_start;
-        if (g_give_up) *l.flow.err = g_give_up, g_give_up = 0;
+        if (g_give_up) *l.flow.err = l.flow.err_tag | g_give_up, g_give_up = 0;
     }
     g_launches.push_back(l);
     return cudaSuccess;

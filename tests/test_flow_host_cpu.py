@@ -174,3 +174,20 @@ def test_a_wait_given_up_with_pageable_outputs(dev):
     assert dev.decode(code, 24 * 211, host_out=True, **big) == OK
     assert dev.decode(code, 24 * 211, **big) == OK
     dev.c.ldpc_code_destroy(code)
+
+
+def test_a_wait_given_up_in_the_fixed_scratch(dev):
+    """The allocation-free decode's time-out is told by the next such call on the same code, not on another."""
+    codes = [dev.code(4, 24, 150) for _ in range(2)]
+    N = 24 * 150
+    call = dict(gamma=32, max_iter=30, early_stop=1, noalloc=True)
+    for code in codes:
+        assert dev.decode(code, N, **call) == OK and form(dev) == "flow"
+        dev.c.fake_give_up(1)
+        assert dev.decode(code, N, **call) == OK
+    assert dev.decode(codes[0], N, gamma=32, max_iter=30) == OK  # ldpc_decode has its own
+    for code in codes:
+        assert dev.decode(code, N, **call) == ETIMEOUT
+        assert dev.decode(code, N, **call) == OK
+    for code in codes:
+        dev.c.ldpc_code_destroy(code)
