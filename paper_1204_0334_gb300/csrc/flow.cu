@@ -48,26 +48,32 @@
 #include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <map>
 #include <mutex>
 #include <new>
-#include <unordered_map>
+#include <utility>
 
 namespace ldpc {
 namespace flow {
 
 int resident_blocks(const void *kernel, size_t smem) {
     static std::mutex mu;
-    static std::unordered_map<const void *, int> blocks;
-    std::lock_guard<std::mutex> lk(mu);
-    auto f = blocks.find(kernel);  // each kernel has one shared-memory size
-    if (f != blocks.end()) return f->second;
+    static std::map<std::pair<int, const void *>, int> blocks;  // by device (each has to be asked for the memory)
     int dev = 0, sms = 0, bps = 0;
     cudaGetDevice(&dev);
+    std::lock_guard<std::mutex> lk(mu);
+    const auto key = std::make_pair(dev, kernel);
+    auto f = blocks.find(key);  // each kernel has one shared-memory size
+    if (f != blocks.end()) return f->second;
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
     cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&bps, kernel, kThreads, smem);
     cudaGetLastError();
-    return blocks[kernel] = bps * sms;
+    try {
+        blocks.emplace(key, bps * sms);
+    } catch (const std::bad_alloc &) {
+    }
+    return bps * sms;
 }
 
 // rows and variables of a tile by the code's degrees and the storage (as Cfg in flow.cuh)

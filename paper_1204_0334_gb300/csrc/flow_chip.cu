@@ -23,7 +23,8 @@
 #include <cstring>
 #include <map>
 #include <mutex>
-#include <utility>
+#include <new>
+#include <tuple>
 
 namespace ldpc {
 namespace chip {
@@ -49,16 +50,19 @@ static int most_lines(const Code &c, int V, int P, bool early) {
 
 int pick(const void *kernel, const Code &c, int V, bool ms, const ChipArgs &a, int P) {
     static std::mutex mu;
-    static std::map<std::pair<const void *, int>, int> active;  // clusters resident at once, one block an SM
+    // clusters resident at once, one block an SM, by device, kernel and blocks of a cluster
+    static std::map<std::tuple<int, const void *, int>, int> active;
+    int dev = 0, E = 0;
+    cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mu);
-    int E = 0;
     for (int i = 0; i < c.J * c.L; ++i) E += c.sh[i] >= 0 ? c.p : 0;
     for (int C = 16; C >= 1; C /= 2) {
         const int NC = (c.N + C - 1) / C;
         if (bytes(c, V, ms, a.want_post, NC) > kChipMost || (!a.any && E > C * most_lines(c, V, P, a.early))) return 0;  // fewer blocks hold less
         if ((C - 1) * NC >= c.N) continue;  // a block would have no variable
-        const auto key = std::make_pair(kernel, C);
-        auto f = active.find(key);
+        const auto key = std::make_tuple(dev, kernel, C);
+        const auto f = active.find(key);
+        int n = f == active.end() ? 0 : f->second;
         if (f == active.end()) {
             cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kChipMost);
             cudaFuncSetAttribute(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -72,14 +76,16 @@ int pick(const void *kernel, const Code &c, int V, bool ms, const ChipArgs &a, i
             at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
             cfg.attrs = at;
             cfg.numAttrs = 1;
-            int n = 0;
             if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
                 cudaGetLastError();
                 n = 0;
             }
-            f = active.emplace(key, n).first;
+            try {
+                active.emplace(key, n);
+            } catch (const std::bad_alloc &) {
+            }
         }
-        if (P <= f->second) return C;
+        if (P <= n) return C;
     }
     return 0;
 }

@@ -352,22 +352,26 @@ __device__ __forceinline__ uint32_t load_if(const uint32_t *p, bool on) {
 }
 
 // blocks of a persistent launch: resident blocks per SM (occupancy API, cached per
-// kernel and dynamic shared-memory size) times the SM count; also raises the kernel's
+// device, kernel and dynamic shared-memory size) times the SM count; also raises the kernel's
 // dynamic shared-memory limit to the largest size requested so far
 template <typename K>
 int persistent_blocks(K kernel, size_t smem) {
     static std::mutex mu;
-    static std::unordered_map<const void *, size_t> limit;         // kernel -> attribute set
-    static std::unordered_map<const void *, std::unordered_map<size_t, int>> cache;  // -> blocks per SM
-    static int sms = 0;
+    struct Device {
+        int sms = 0;
+        std::unordered_map<const void *, size_t> limit;         // kernel -> attribute set
+        std::unordered_map<const void *, std::unordered_map<size_t, int>> cache;  // -> blocks per SM
+    };
+    static std::unordered_map<int, Device> devices;  // each has to be asked for the memory
+    int dev = 0;
+    cudaGetDevice(&dev);
     std::lock_guard<std::mutex> lk(mu);
+    auto &[sms, limit, cache] = devices[dev];
     const void *key = (const void *)kernel;
     auto &per = cache[key];
     auto f = per.find(smem);
     if (f != per.end()) return f->second * sms;
     if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
         cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
         if (sms <= 0) sms = 1;
     }

@@ -191,3 +191,17 @@ def test_a_wait_given_up_in_the_fixed_scratch(dev):
         assert dev.decode(code, N, **call) == OK
     for code in codes:
         dev.c.ldpc_code_destroy(code)
+
+
+def test_a_second_device(dev):
+    """What a kernel may have and how many of its blocks fit are asked for on each device: the first call of
+    every form on a second device, after the same calls on the first."""
+    for d in (0, 1):
+        dev.c.fake_device(d)
+        code, long = dev.code(3, 6, 64), dev.code(4, 24, 211)
+        assert dev.decode(code, 384, 32, max_iter=30) == 0 and form(dev) == "chip"
+        assert dev.decode(code, 384, 8192, max_iter=30) == 0 and form(dev) == "launches"
+        assert dev.decode(long, 24 * 211, 4096, max_iter=30) == 0 and form(dev) == "flow"
+        assert dev.c.fake_refused() == 0
+        dev.c.ldpc_code_destroy(code)
+        dev.c.ldpc_code_destroy(long)
