@@ -301,7 +301,8 @@ ldpc_status ldpc_ber_sim(ldpc_code code, double ebn0_db, uint64_t seed, uint64_t
 /*
  * ldpc_tune_slots -- the autotuner of the continuous simulation's slot count Gamma
  * (no paper counterpart; the paper fixes Gamma = 32 for its GPU, Sec. IV-A).  Times
- * ldpc_ber_sim's decoding at 16384, 8192, 4096, 2048 and 1024 slots (a settling run
+ * ldpc_ber_sim's decoding by a launch per pass, the form that runs to an error target
+ * take and whose speed the slots decide, at 16384, 8192, 4096, 2048 and 1024 slots (a settling run
  * of one frame per slot, then a timed run of four frames per slot, frames drawn from
  * the reserved id range [2^63, 2^63 + 2^43), which the caller's runs should avoid) and
  * keeps the fastest in the code object for opts->algo / opts->msg.

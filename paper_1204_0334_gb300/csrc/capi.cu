@@ -510,12 +510,13 @@ ldpc_status ldpc_tune_slots(ldpc_code c, double ebn0_db, uint64_t seed, const ld
     for (int i = 0; i < kTuneCands; ++i) {
         const int slots = kTuneSlots[i];
         // frames of a reserved id range (top bit set): a short run to settle the workspace and
-        // caches, then the timed run of four frames per slot
+        // caches, then the timed run of four frames per slot; by launches, the form whose speed the
+        // slots decide (the flow decoder keeps what fits in L2 in work, whatever their number)
         const uint64_t base = (1ull << 63) + (uint64_t)i * (1ull << 40);
-        st = qc_ber_sim_refill(c, sigma, seed, base, slots, 1ll << 60, slots, o, h, s);
+        st = qc_ber_sim_refill(c, sigma, seed, base, slots, 1ll << 60, slots, o, h, s, nullptr, true);
         if (st != LDPC_OK) return st;
         const auto t0 = std::chrono::steady_clock::now();
-        st = qc_ber_sim_refill(c, sigma, seed, base + (1ull << 39), 4ll * slots, 1ll << 60, slots, o, h, s);
+        st = qc_ber_sim_refill(c, sigma, seed, base + (1ull << 39), 4ll * slots, 1ll << 60, slots, o, h, s, nullptr, true);
         if (st != LDPC_OK) return st;
         const double sec = std::chrono::duration<double>(std::chrono::steady_clock::now() - t0).count();
         const double rate = sec > 0 ? (double)h[0] * K / sec / 1e6 : 0.0;

@@ -175,9 +175,10 @@ struct StreamIO {
     uint8_t *hard;
     int32_t *iters, *ok;
 };
+// by_launches: a launch a pass on gamma slots, also where the flow decoder would take the run
 ldpc_status qc_ber_sim_refill(ldpc_code c, double sigma, uint64_t seed, uint64_t first_frame, int64_t max_frames,
                               int64_t target, int gamma, const ldpc_decode_opts &o, unsigned long long *h,
-                              cudaStream_t s, const StreamIO *io = nullptr);
+                              cudaStream_t s, const StreamIO *io = nullptr, bool by_launches = false);
 
 // systematic encoder (encode.cu)
 void enc_free(ldpc_encoder_s *e);

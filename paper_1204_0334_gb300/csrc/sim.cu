@@ -460,11 +460,11 @@ stream_out_kernel(const uint32_t *__restrict__ hw, const uint32_t *__restrict__ 
 // counted (sigma, seed, first_frame and target are unused).
 ldpc_status qc_ber_sim_refill(ldpc_code c, double sigma, uint64_t seed, uint64_t first_frame, int64_t max_frames,
                               int64_t target, int gamma, const ldpc_decode_opts &o, unsigned long long *h,
-                              cudaStream_t s, const StreamIO *io) {
+                              cudaStream_t s, const StreamIO *io, bool by_launches) {
     // one launch where the frames' results do not depend on how many are in flight: a frame-error target
     // that cannot be met (or a caller's batch), all-zero codewords, one rule for every frame
-    if (o.algo != LDPC_ALGO_NOMS && flow_sim_pays(c->d, gamma, o) && (io || (o.codewords == LDPC_CODEWORDS_ZERO && target > max_frames)))
-    {
+    if (!by_launches && o.algo != LDPC_ALGO_NOMS && flow_sim_pays(c->d, gamma, o) &&
+        (io || (o.codewords == LDPC_CODEWORDS_ZERO && target > max_frames))) {
         const ldpc_status e = flow_sim_code(c, sigma, seed, first_frame, max_frames, gamma, o, h, s, io);
         if (e != LDPC_ENOMEM || (size_t)gamma > c->ws.gamma_cap) return e;
     }

@@ -54,6 +54,9 @@ class FakeDevice:
     def calls(self, name):
         return self.c.fake_calls(name.encode())
 
+    def opts(self, **kw):
+        return pkg.default_opts(**kw)
+
     def decode(self, code, N, gamma, *, noalloc=False, post=False, host_out=False, **opts):
         """ldpc_decode (or _noalloc) on device buffers, the decisions to the host with host_out; the status"""
         o = pkg.default_opts(**opts)

@@ -205,3 +205,18 @@ def test_a_second_device(dev):
         assert dev.c.fake_refused() == 0
         dev.c.ldpc_code_destroy(code)
         dev.c.ldpc_code_destroy(long)
+
+
+@pytest.mark.parametrize("algo,msg", [(0, 0), (0, 1), (1, 2)])
+def test_tuner_times_the_form_that_the_slots_decide(dev, algo, msg):
+    """The slot count's candidates are timed as the runs that it decides are run: by launches on that many
+    slots, where the flow decoder keeps the same few packages in work at every candidate."""
+    import ctypes
+
+    code = dev.code(4, 24, 40)
+    o = dev.opts(max_iter=5, early_stop=1, algo=algo, msg=msg)
+    picked = ctypes.c_int32()
+    assert dev.c.ldpc_tune_slots(code, 2.0, 1, ctypes.byref(o), ctypes.byref(picked), None, None) == 0
+    assert not dev.flows() and sum("sim_check_kernel" in n for n in dev.names()) >= 10
+    assert dev.sim(code, 500, 64, algo=algo, msg=msg, early_stop=1) == 0 and len(dev.flows()) == 1
+    dev.c.ldpc_code_destroy(code)
