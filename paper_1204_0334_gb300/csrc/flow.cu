@@ -223,6 +223,15 @@ bool flow_pays(const QcDesc &d, int gamma, const ldpc_decode_opts &o) {
     return o.early_stop ? !shortcode || lines < 60000 : !shortcode && lines > 80000;
 }
 
+// Frames of one launch: it holds every SM until it ends, so its edges times frames times iterations are
+// bounded (2^39: 1.4 s at the 3.9e11 a second of n = 18360, FP32, 30 iterations; 249525 frames of that, so
+// what is lost where one launch ends and the next begins, under a millisecond, does not show), but every lane
+// in flight gets a frame.
+static int64_t launch_frames(const QcDesc &d, int max_iter, int64_t lanes) {
+    const int64_t work = std::max<int64_t>(1, (int64_t)d.E * max_iter);
+    return std::min<int64_t>((int64_t)1 << 20, std::max(((int64_t)1 << 39) / work, lanes));
+}
+
 // a launch on W slots of m: the code's entry, the buffers, the options
 static ldpc_status prepare(const QcDesc &d, const FlowMem &m, const ldpc_decode_opts &o, int W, bool post, Start &st, Args &a,
                            uint32_t *tiles) {
@@ -271,16 +280,24 @@ ldpc_status flow_decode(const QcDesc &d, const FlowMem &m, const float *llr, int
     uint32_t tiles = 0;
     const ldpc_status e = prepare(d, m, o, std::min(m.W, P), post != nullptr, st, a, &tiles);
     if (e != LDPC_OK) return e;
-    Code &c = st.code;
-    c.gamma = gamma;
-    c.llr = llr, c.post = post, c.hard = hard, c.iters = iters, c.ok = ok;
-    a.P = P;
     // with several long packages in work a phase of its own for the syndrome costs no time and saves the
     // check step of a package that has stopped; with few, or short ones, it would add its latency to
     // every iteration (4 x 8, p = 100, 256 frames, FP16: 537 us with, launches 445)
     a.split = a.early && a.W >= 4 && d.E >= kShortCode;
     st.tiles = (d.N + outv(d.J) - 1) / outv(d.J);
-    return run(d, o, a, st, tiles, s);
+    Code &c = st.code;
+    const int W = a.W, most = (int)(launch_frames(d, o.max_iter, (int64_t)W * 32 * V) / (32 * V));  // packages a launch
+    for (int at = 0; at < P; at += most) {
+        const size_t f0 = (size_t)at * 32 * V;
+        a.P = std::min(most, P - at);
+        a.W = std::min(W, a.P);
+        c.gamma = (int)std::min<size_t>(gamma - f0, (size_t)a.P * 32 * V);
+        c.llr = llr + f0 * d.N, c.post = post ? post + f0 * d.N : nullptr, c.hard = hard ? hard + f0 * d.N : nullptr;
+        c.iters = iters ? iters + f0 : nullptr, c.ok = ok ? ok + f0 : nullptr;
+        const ldpc_status r = run(d, o, a, st, tiles, s);
+        if (r != LDPC_OK) return r;
+    }
+    return LDPC_OK;
 }
 
 }  // namespace ldpc
@@ -409,8 +426,8 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
     ldpc_flow_ws &w = *c->flow;
     const FlowMem m{w.buf[0], w.buf[1], w.buf[2], w.buf[3], w.buf[4], W, w.log_cap, w.err, 0};
     std::memset(h, 0, 8 * sizeof(*h));
-    constexpr int64_t kMost = (int64_t)1 << 20;  // frames a launch, so that none runs for minutes
-    for (int64_t at = 0; at < max_frames; at += kMost) {
+    const int64_t most = launch_frames(c->d, o.max_iter, (int64_t)W * 32 * V);
+    for (int64_t at = 0; at < max_frames; at += most) {
         Start st;
         Args a;
         uint32_t tiles = 0;
@@ -421,7 +438,7 @@ ldpc_status flow_sim_code(ldpc_code c, double sigma, uint64_t seed, uint64_t fir
         static_assert(sizeof(Sim) <= 512, "room before the slots");
         st.tiles = st.code.nsyn;
         Sim &si = st.sim;
-        si.limit = (unsigned long long)std::min(kMost, max_frames - at);
+        si.limit = (unsigned long long)std::min(most, max_frames - at);
         si.first = (io ? 0ull : first_frame) + (unsigned long long)at;
         si.seed = seed;
         si.sigma = (float)sigma;

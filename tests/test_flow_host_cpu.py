@@ -220,3 +220,33 @@ def test_tuner_times_the_form_that_the_slots_decide(dev, algo, msg):
     assert not dev.flows() and sum("sim_check_kernel" in n for n in dev.names()) >= 10
     assert dev.sim(code, 500, 64, algo=algo, msg=msg, early_stop=1) == 0 and len(dev.flows()) == 1
     dev.c.ldpc_code_destroy(code)
+
+
+@pytest.mark.parametrize("J,L,p,max_iter,frames", [(4, 24, 765, 30, 1 << 20), (4, 24, 4200, 100, 1 << 20),
+                                                   (3, 6, 64, 30, 3 << 20), (4, 24, 765, 30, 131072),
+                                                   (4, 8, 300000, 50, 4000)])
+def test_simulation_launches_are_bounded_in_work(dev, J, L, p, max_iter, frames):
+    """A launch holds every SM until it ends: edges x frames x iterations of one stay below 2^39, about a
+    second, whatever the code and the iterations, unless that would leave lanes without a frame."""
+    code = dev.code(J, L, p)
+    assert dev.sim(code, frames, 1024, max_iter=max_iter, early_stop=1) == 0
+    flows = dev.flows()
+    assert sum(f["frames"] for f in flows) == frames
+    for f in flows:
+        assert f["frames"] * J * L * p * max_iter <= 1 << 39 or f["frames"] <= 32 * f["W"]
+    if frames == 131072:
+        assert len(flows) == 1
+    dev.c.ldpc_code_destroy(code)
+
+
+def test_decode_launches_are_bounded_in_work(dev):
+    code = dev.code(4, 24, 765)
+    for kw, n in ((dict(gamma=4001, max_iter=100000), 16), (dict(gamma=2048, max_iter=30), 1)):
+        at = len(dev.flows())
+        assert dev.decode(code, 18360, post=True, **kw) == 0
+        flows = dev.flows()[at:]
+        assert len(flows) > 15 if n > 1 else len(flows) == 1
+        assert sum(f["frames"] for f in flows) == kw["gamma"]
+        for f in flows:
+            assert f["frames"] * 73440 * kw["max_iter"] <= 1 << 39 or f["frames"] <= 32 * f["W"]
+    dev.c.ldpc_code_destroy(code)

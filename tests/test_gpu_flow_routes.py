@@ -81,3 +81,27 @@ def test_captured_decodes(pkg):
         assert torch.equal(a, b)
     for a, b in zip(whole[1:], other.decode(mu, max_iter=6)[1:]):
         assert torch.equal(a, b)
+
+
+@pytest.mark.parametrize("post,frames,gamma", [(True, 8000, None), (False, 9001, None), (False, 9001, 512)])
+def test_several_launches_for_one_call(pkg, post, frames, gamma):
+    """A decode (in a batch, and streamed) and a simulation whose iteration limit allows more work than one
+    launch may hold the chip for give what the same frames give with a lower limit, which none of them reaches."""
+    code = pkg.QCCode(synth.qc_shifts(4, 24, 765, seed=2), 765)
+    if gamma is None:
+        mu = code.channel(3.5, 7, 0, frames)
+        one, n1 = launches(pkg, lambda: code.decode(mu, max_iter=60, early_stop=True, want_post=post))
+        many, n = launches(pkg, lambda: code.decode(mu, max_iter=2000, early_stop=True, want_post=post))
+        part = 2 ** 39 // (73440 * 2000)  # frames of a launch; whole packages in a batch
+        assert int(one[2].max()) < 60 and n1 == 2 and n == 2 * -(-frames // (part // 32 * 32 if post else part))
+        for a, b in zip(one, many):
+            assert a is b is None or torch.equal(a, b)
+    else:
+        def sim(max_iter):
+            r, n = launches(pkg, lambda: code.ber_sim(3.5, seed=7, max_frames=frames, target_frame_errors=1 << 40,
+                                                      gamma=gamma, max_iter=max_iter, early_stop=1))
+            r.pop("seconds")
+            return r, n
+
+        one, many = sim(60), sim(2000)
+        assert one[1] == 2 and many[1] == 6 and one[0] == many[0] and one[0]["frame_errors"] == 0
