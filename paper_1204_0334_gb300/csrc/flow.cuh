@@ -713,21 +713,24 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
             pl.loaded = true;
         }
         const int at = (int)(pl.n - pl.first);
-        pl.e0 = __shfl_sync(0xffffffffu, pl.w0, at);
         pl.e1 = __shfl_sync(0xffffffffu, pl.w1, at);
-        const int is = entry_is(pl.e0, pl.e1, pl.n);
+        int is = entry_is(pl.e1, pl.n);
         if (is == kEntryHere) {
-            if (bits(pl.e0, 0, 3) == F_EXIT) return false;
-            const uint32_t base = bits(pl.e1, kLogTiles, kLogBase);
+            const uint32_t base = bits(pl.e1, kLogTiles, kLogBase), tiles = bits(pl.e1, 0, kLogTiles);
             const uint32_t i = blockIdx.x >= base ? blockIdx.x - base : blockIdx.x + gridDim.x - base;
-            if (i < bits(pl.e1, 0, kLogTiles)) {
+            if (i >= tiles && tiles) {
+                ++pl.n;  // none of its tiles is this block's
+                continue;
+            }
+            pl.e0 = __shfl_sync(0xffffffffu, pl.w0, at);
+            if (entry_whole(pl.e0, pl.n)) {
+                if (!tiles) return false;  // F_EXIT
                 __threadfence();  // the phase's inputs were written before it was opened
                 idx = i;
                 pl.idx = i + gridDim.x;
                 return true;
             }
-            ++pl.n;  // none of its tiles is this block's
-            continue;
+            is = kEntryAhead;
         }
         if (is == kEntryPast) {
             ++pl.n;  // overwritten: it had no tile of this block's (log_entries)

@@ -65,14 +65,15 @@ __host__ __device__ inline unsigned long long entry_w1(uint32_t seq, int slot, u
     x = x << kLogBase | base;
     return x << kLogTiles | tiles;
 }
-// what two words read in entry n's place are: entry n, a later one that has overwritten it, or not (both of)
-// entry n yet
+// what a second word read in entry n's place is: entry n's, a later one's that has overwritten it, or an earlier
 enum { kEntryHere = 0, kEntryPast, kEntryAhead };
-__host__ __device__ inline int entry_is(unsigned long long w0, unsigned long long w1, uint32_t n) {
+__host__ __device__ inline int entry_is(unsigned long long w1, uint32_t n) {
     const uint32_t ahead = ((uint32_t)(w1 >> (kLogTiles + kLogBase + kLogSlot)) - n) & kLogMask;
-    if (ahead == 0u)
-        return (uint32_t)(w0 >> (4 + kLogIt + kLogPk)) == (n & kLogMask) >> kLogLow ? kEntryHere : kEntryAhead;
-    return ahead < (kLogMask >> 1) ? kEntryPast : kEntryAhead;
+    return ahead == 0u ? kEntryHere : ahead < (kLogMask >> 1) ? kEntryPast : kEntryAhead;
+}
+// whether the first word read beside it is entry n's too
+__host__ __device__ inline bool entry_whole(unsigned long long w0, uint32_t n) {
+    return (uint32_t)(w0 >> (4 + kLogIt + kLogPk)) == (n & kLogMask) >> kLogLow;
 }
 
 // Entries of the phase log, a power of two.  Entry n is overwritten by entry n + length, which must not be

@@ -105,10 +105,11 @@ void fake_flow(int i, long long *x) {
 }
 
 // what a block makes of a log entry's place where it finds the words written for entries n0 and n1 and looks
-// for entry n (entry_is); kind, package and slot of the entries: their numbers
+// for entry n, with a tile of its own (entry_is, entry_whole); kind, package and slot of the entries: their numbers
 int fake_entry_is(unsigned n0, unsigned n1, unsigned n) {
-    return ldpc::flow::entry_is(ldpc::flow::entry_w0(n0, (int)(n0 % 7), 1, 99999, (int)(n0 & 0x3ffffff)),
-                                ldpc::flow::entry_w1(n1, (int)(n1 & 255), n1 % 152, n1 & 0xffffff), n);
+    const int is = ldpc::flow::entry_is(ldpc::flow::entry_w1(n1, (int)(n1 & 255), n1 % 152, n1 & 0xffffff), n);
+    const auto w0 = ldpc::flow::entry_w0(n0, (int)(n0 % 7), 1, 99999, (int)(n0 & 0x3ffffff));
+    return is == ldpc::flow::kEntryHere && !ldpc::flow::entry_whole(w0, n) ? (int)ldpc::flow::kEntryAhead : is;
 }
 
 // --- the runtime ---------------------------------------------------------------------------------
