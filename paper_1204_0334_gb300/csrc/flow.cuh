@@ -53,6 +53,7 @@ __device__ __forceinline__ void bulk_wait() {  // all but the last N groups are 
 }
 __device__ __forceinline__ void bulk_wait_read() { asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_async() { asm volatile("fence.proxy.async;" ::: "memory"); }
+__device__ __forceinline__ void fence_async_global() { asm volatile("fence.proxy.async.global;" ::: "memory"); }
 __device__ __forceinline__ void fence_async_shared() { asm volatile("fence.proxy.async.shared::cta;" ::: "memory"); }
 
 __device__ __forceinline__ void ld_entry(const Entry *p, unsigned long long &w0, unsigned long long &w1) {
@@ -726,6 +727,7 @@ __device__ __forceinline__ bool take(const Args &a, int lane, Place &pl, uint32_
             if (entry_whole(pl.e0, pl.n)) {
                 if (!tiles) return false;  // F_EXIT
                 __threadfence();  // the phase's inputs were written before it was opened
+                fence_async_global();  // by other blocks' bulk copies too, and bulk copies read them next
                 idx = i;
                 pl.idx = i + gridDim.x;
                 return true;
