@@ -152,14 +152,17 @@ ldpc_status ldpc_decode(ldpc_code code, const float *llr, int32_t gamma, const l
  * cudaMalloc, or processes whose device memory is reserved up front by another
  * allocator).  The paper has no counterpart.  Same arguments and results as
  * ldpc_decode, but every buffer must be device memory and the decoder's
- * workspace comes from a fixed 16 MiB array inside the library (held on every
+ * workspace comes from a fixed 16 MiB array inside the library, and a second
+ * one of 1.1 MB for what the one-launch form schedules by (both held on every
  * GPU that loads it until the process exits); the call itself calls no
  * cudaMalloc/cudaFree.  A decode of gamma frames needs about
  * (4E + 8N + N/8) * gamma bytes (rounded up to 128 frames): requests beyond
  * the array return LDPC_EINVAL with the size in ldpc_last_error().  The first
- * call on a device looks up the array's device address (cudaGetSymbolAddress)
- * with that device current; make that first call before any stream capture.
- * All calls share the array, and each decode initializes what it reads, but
+ * call on a device looks up the arrays' device addresses (cudaGetSymbolAddress)
+ * with that device current and takes 4 KB of pinned host memory, kept until the
+ * process exits, in which the device reports a wait that gave up; make that
+ * first call before any stream capture.
+ * All calls share the arrays, and each decode initializes what it reads, but
  * calls whose GPU work overlaps (other streams or threads) race on it.
  * Sum-product (F32/F16 storage) and integer min-sum; LDPC_EUNSUPPORTED for NOMS.
  */
@@ -427,7 +430,9 @@ ldpc_status ldpc_phi_eval(const float *x, float *y, int64_t n, int32_t variant, 
  * totals, Sec. V).  While enabled, each check-node and variable-node kernel
  * launch of the block-code decoder is bracketed by CUDA events on its own
  * stream.  ldpc_profile_read synchronizes those events and returns the summed
- * device time per kind.  `launches` counts every kernel this library has
+ * device time per kind.  A decode or a simulation that runs as one launch (see
+ * ldpc_decode) has no such launches: it adds nothing to the counts and times
+ * per kind, only to `launches`; time it as a whole.  `launches` counts every kernel this library has
  * launched since the last ldpc_profile_enable call, enabled or not.
  * Not thread-safe; enable/read from the thread that issues the decodes.
  */

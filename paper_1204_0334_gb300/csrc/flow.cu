@@ -28,19 +28,22 @@
 //
 // Three stages of 72 KB: a tile arrives while another is computed and a third leaves.  What bounds it
 // (n = 18360, FP32, 2048 frames, 30 iterations): the compute warps, 5500 cycles a check tile and 3600
-// a variable tile of the 5400 a tile takes on average (about 50 instructions per edge and iteration,
-// 81 in the launches before).  15.2 ms before, 11.5 ms now; the n = 15168 integer min-sum with early
-// stop, 4096 frames: 3.18 -> 1.92 ms; 40 frames of the n = 18360 code with early stop: 749 -> 250 us
-// (the launches of all 30 iterations are gone); an irregular n = 2532 code, 1000 frames: 886 -> 366 us.
+// a variable tile of the 5400 a tile takes on average (66 warp instructions per edge and iteration in all,
+// the waiting warps' among them, at 65 % of the issue slots; 1.4 TB/s of the lines are written back to HBM
+// although they are read from L2).  15.2 ms before, 11.6 now; the n = 15168 integer min-sum with early
+// stop, 4096 frames: 3.18 -> 1.90 ms; 40 frames of the n = 18360 code with early stop: 749 -> 250 us
+// (the launches of all 30 iterations are gone); an irregular n = 2532 code, 1000 frames: 886 -> 375 us.
+//
+// A launch holds every SM until it ends, so long calls are several launches (launch_frames).
 //
 // Refill mode (the simulation with a frame-error target that cannot be met, and the streaming decode):
 // every lane of a slot is a frame slot.  A step of a package is three phases: the syndrome, after which
 // frames leave and the next ones enter; the check step with tiles that count wrong bits (or write
 // decision rows) and tiles that draw (or read) the new frames' channel LLRs into the slot's lines; the
 // variable step.  As many slots as L2 holds give the same counts as the caller's number of slots, since
-// a frame's result does not depend on the others.  n = 18360, 32768 frames at 3.5 dB: FP32 68.4 -> 59.8
-// ms, FP16 59.8 -> 48.5 ms; the chip computes 78 % of the time (FP32), the rest is the phases' latency at
-// the eight packages that fit.
+// a frame's result does not depend on the others.  n = 18360, 32768 frames at 3.5 dB: FP32 68.4 -> 58.9
+// ms, FP16 59.8 -> 47.5 ms; the compute warps have a tile 78 % of the time (FP32), the rest is the phases'
+// latency at the eight packages that fit.
 //
 // The arithmetic is that of the pass kernels (qc_pipe.cu), operation by operation.
 #include "flow_internal.cuh"

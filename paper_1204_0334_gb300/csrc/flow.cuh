@@ -230,7 +230,7 @@ __device__ __forceinline__ void noms_row(uint32_t pm, float clip, const float2 *
     }
 }
 
-// check tile: compute warp `warp` takes rows warp, warp + 8, ... of the tile, in place
+// check tile: compute warp `warp` takes rows warp, warp + 24, ... of the tile, in place
 template <typename C, int DC, int V, int RULE, bool REG>
 __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp, int lane, float clip,
                                         const float2 *__restrict__ prm) {
@@ -328,7 +328,7 @@ __device__ __forceinline__ void cn_tile(uint32_t *stage, const Desc &d, int warp
     }
 }
 
-// variable tile: warp `warp` takes variables warp, warp + 8, ...; beta (or its transform) in place,
+// variable tile: warp `warp` takes variables warp, warp + 24, ...; beta (or its transform) in place,
 // decision words and posteriors to global memory
 template <typename C, int JX, int V, int RULE, bool REG>
 __device__ __forceinline__ void vn_tile(uint32_t *stage, const uint32_t *hwold, const Desc &d, int warp, int lane,

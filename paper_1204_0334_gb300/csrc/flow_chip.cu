@@ -12,8 +12,8 @@
 // The blocks of a cluster are as many as leave all packages resident at once (16, 8, 4, 2 or 1): more
 // blocks a package, fewer rows a warp.  What bounds it is latency: the chain of a row (its remote loads
 // in flight together, then the sums and transforms) and the barriers.  n = 384, 32 frames, 30 iterations:
-// 283 us by launches, 86 here
-// (3500 cycles an iteration in the check step and its barrier, 2300 in the variable step and its own).
+// 283 us by launches, 82 to 86 here (it differs from process to process; 3500 cycles an iteration in the
+// check step and its barrier, 2300 in the variable step and its own).
 //
 // The arithmetic is that of the pass kernels (qc_pipe.cu), operation by operation.
 #include "flow_internal.cuh"
