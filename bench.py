@@ -43,13 +43,18 @@ METRIC = "decoded info Mbit/s (n=18360, 30 iters) at BER matching FP64 oracle"
 # sources hash the same (null as soon as a kernel changes, until re-measured).
 CN_DRAM_BYTES_PER_LAUNCH = {"f32": (2277.8e6, "f63b990e626641ef")}
 KERNEL_SOURCES = ("qc_pipe.cu", "qc_device.cuh", "ldpc_internal.cuh")
+# The same for the flow decoder's kernel, which runs the whole step: executed warp instructions
+# (smsp__inst_executed.sum, all warps) and DRAM bytes per edge line and iteration, from one ncu run of 32768
+# frames of that workload (profiles/kernels_of_the_cases.md).
+FLOW_PER_LINE = {"f32": (80.91, 377.1, "bcfb70f2bf8da17b")}
+FLOW_SOURCES = ("flow.cuh", "flow_internal.cuh", "flow.cu", "qc_device.cuh", "ldpc_internal.cuh")
 
 
-def kernel_source_hash() -> str:
+def kernel_source_hash(files=KERNEL_SOURCES) -> str:
     import hashlib
 
     h = hashlib.sha256()
-    for f in KERNEL_SOURCES:
+    for f in files:
         with open(os.path.join(ROOT, "paper_1204_0334_gb300", "csrc", f), "rb") as fh:
             h.update(fh.read())
     return h.hexdigest()[:16]
@@ -346,19 +351,31 @@ def run_ours(a):
     peaks = load_peaks()
     peak = peaks.get("hbm_gbs", 6800.0)
     path_gbs = (4 * E_EDGES * s_msg + N_BITS * s_mu + N_BITS / 8) * local_iters / (ms / 1e3) / 1e9
-    # the whole step is one kernel that keeps its messages in L2 (flow.cu); without separate check passes
-    # the roofline figure is the path's canonical message bytes against the HBM rate they no longer take
+    # the whole step is one kernel that reads its messages from L2 (flow.cu) and is bound by its instructions:
+    # those executed against the issue slots of the chip at the sampled clock.  The path's canonical message
+    # bytes per second stay beside it (path_achieved_gbs), a rate of work and not of DRAM traffic.
     fused = prof["cn_launches"] == 0
     rule = "sum-product" if algo == pkg.ALGO_SP else "min-sum"
-    roof = {"bound": "issue" if fused else "hbm",
-            "kernel": f"flow tile_kernel ({rule}, whole path)" if fused else f"cn_pipe_kernel ({rule})",
-            "achieved": path_gbs if fused else cn_bytes / cn_s / 1e9, "peak": peak, "unit": "GB/s",
-            "frac": (path_gbs if fused else cn_bytes / cn_s / 1e9) / peak,
-            "traffic": traffic,
-            "traffic_source": traffic_src,
-            "algorithmic_bytes_per_launch": cn_bytes / prof["cn_launches"] if not fused else None,
-            "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks else "fallback",
-            "cn_launches": prof["cn_launches"], "cn_ms_avg": prof["cn_ms"] / max(1, prof["cn_launches"]),
+    if fused:
+        frames_per_line = {"f32": 32, "f16": 64, "i8": 128}[a.msg]
+        lines = E_EDGES * local_iters / frames_per_line
+        per = FLOW_PER_LINE.get(a.msg)
+        current = per and default_workload and per[2] == kernel_source_hash(FLOW_SOURCES)
+        sms = torch.cuda.get_device_properties(dev).multi_processor_count
+        slots = sms * 4 * clk["sm_mhz"] / 1e3 if clk.get("sm_mhz") else None
+        rate = per[0] * lines / (ms / 1e3) / 1e9 if current else None
+        roof = {"bound": "issue", "kernel": f"flow tile_kernel ({rule}, whole path)", "achieved": rate, "peak": slots,
+                "unit": "Ginst/s", "frac": rate / slots if rate and slots else None,
+                "traffic": per[1] * lines / a.steps if current else None,
+                "traffic_source": f"ncu, DRAM bytes per edge line and iteration, sources {per[2]}" if current else
+                "no ncu measurement of this kernel source and workload",
+                "algorithmic_bytes_per_launch": None, "peak_source": "4 issue slots per SM and cycle, sampled clock"}
+    else:
+        roof = {"bound": "hbm", "kernel": f"cn_pipe_kernel ({rule})", "achieved": cn_bytes / cn_s / 1e9, "peak": peak,
+                "unit": "GB/s", "frac": cn_bytes / cn_s / 1e9 / peak, "traffic": traffic,
+                "traffic_source": traffic_src, "algorithmic_bytes_per_launch": cn_bytes / prof["cn_launches"],
+                "peak_source": "measured (MEASURED_PEAKS.json hbm_gbs)" if "hbm_gbs" in peaks else "fallback"}
+    roof |= {"cn_launches": prof["cn_launches"], "cn_ms_avg": prof["cn_ms"] / max(1, prof["cn_launches"]),
             "vn_ms_avg": prof["vn_ms"] / max(1, prof["vn_launches"]),
             "path_bytes_per_frame_iter": 4 * E_EDGES * s_msg + N_BITS * s_mu + N_BITS // 8,
             "path_achieved_gbs": path_gbs}
@@ -368,8 +385,9 @@ def run_ours(a):
             "config": {"workload": workload_name(a), "slots": a.gamma, "frames_per_step": a.frames,
                        "iters_cap": a.iters,
                        "early_stop": not a.no_early_stop, "ebn0_db": a.ebn0, "msg": a.msg,
-                       "l2": "inputs larger than L2 (message store %.2f GB)" % (
-                           E_EDGES * s_msg * a.gamma / 1e9)},
+                       "l2": "inputs larger than L2 (%.2f GB of channel LLRs drawn and decoded per step%s)" % (
+                           4 * N_BITS * a.frames / 1e9,
+                           "; the packages in work are kept in L2" if fused else "")},
             "frames": frames, "mean_iters": iters_sum / frames, "fer": fe / frames, "ber": be / (frames * N_BITS),
             "frames_per_s": frames / (ms / 1e3), "roofline": roof, "clocks": clk,
             "gpu_launches": prof["launches"]}
