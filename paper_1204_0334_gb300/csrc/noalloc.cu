@@ -7,12 +7,15 @@
 // fully reserved up front by another allocator.  For them the decoder's
 // workspace lives in a fixed array compiled into this library (kNoallocBytes,
 // 16 MiB, resident on every GPU that loads the library until the process
-// exits).  The caller still passes its device input and output buffers.
+// exits).  The caller still passes its device input and output buffers.  A
+// second array of 1.1 MB holds what the flow decoder schedules by.
 //
-// The array is a static __device__ object of this file.  In host code its name
-// is only a host-side stand-in, so its device address is looked up once per
-// device with cudaGetSymbolAddress (on the first call made with that device
-// current) and handed to the kernels as a plain pointer.
+// The arrays are static __device__ objects of this file.  In host code their
+// names are only host-side stand-ins, so their device addresses are looked up
+// once per device with cudaGetSymbolAddress (on the first call made with that
+// device current) and handed to the kernels as plain pointers.  That call also
+// allocates the pinned host words in which the flow decoder reports a wait that
+// gave up.
 //
 // Every call uses the same array, which keeps whatever the previous call left:
 // the decode steps initialize everything they read (the flag words and the
